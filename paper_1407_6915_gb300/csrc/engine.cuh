@@ -545,6 +545,15 @@ FDEV void tma_store_3d(const CUtensorMap *tmap, int x, int y, int z, const void 
                  : "memory");
 }
 
+// tma_store_3d for a 4-D map, at (x, y, z, w)
+FDEV void tma_store_4d(const CUtensorMap *tmap, int x, int y, int z, int w, const void *src)
+{
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                     reinterpret_cast<uint64_t>(tmap)),
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(src))
+                 : "memory");
+}
+
 // wait until every committed bulk copy of this thread has completed its writes
 FDEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 

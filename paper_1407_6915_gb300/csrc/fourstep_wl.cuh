@@ -5,9 +5,9 @@
 //   pass A (column DFTs): Yt[j2][k1] = w_n^{j2 k1} sum_{j1} x[j1 N2 + j2] w_{N1}^{j1 k1}
 //   pass B (row DFTs):    X[k1 + N1 k2] = sum_{j2} Yt[j2][k1] w_{N2}^{j2 k2}
 // with Yt in an L2-resident ring of chunk buffers, stored in blocks of the
-// row tiles' W_B rows, [k1 / W_B][j2][k1 mod W_B], so that every row tile is
-// one contiguous block (its TMA load is one region, and once it is consumed
-// its L2 lines are dropped whole); a row tile of segment s
+// row tiles' panels of PW_B rows, [k1 / PW_B][j2][k1 mod PW_B], so that every
+// row tile is one contiguous block (its TMA load is one region, and once it is
+// consumed its L2 lines are dropped whole); a row tile of segment s
 // waits for the column tiles of s, a column tile for the row tiles of the
 // segment that last used its ring slot (per-segment counters).
 //
@@ -21,7 +21,7 @@
 // b = j + P e, e < 32 / P, so it ends with the bins k = j + P m, m < 32.
 // The one exchange between the stages goes through the line's own column of
 // the tile buffer, in place, so a line needs no shared memory beyond its
-// tile.  Two lines are interleaved over each half-warp (8 lanes of each), so
+// tile.  Two lines (WlPass::line_of) share each half-warp (8 lanes of each), so
 // that every shared access of a half-warp touches 16 distinct 8-byte bank
 // pairs; with the TMA swizzle of the tile rows and the exchange's row
 // permutation phi(m) = m ^ ((m >> 5) & 7), every access is conflict-free.  The
@@ -40,9 +40,10 @@
 // taken before it by CTAs that are running: no co-residency is assumed.
 // Per CTA: NB tile buffers, compute warps that run a tile at a time, a loader
 // warp (takes tiles, probes their dependency, issues the TMA loads and, for
-// column tiles, the tile's four-step factors) and a retirer warp (stores row
-// tiles with TMA, drops consumed ring lines from L2, frees buffers, publishes
-// finished tiles on the segment counters in batches).  Every wait is bounded
+// column tiles, the tile's four-step factors) and a retirer warp per buffer
+// (stores column tiles into the ring and row tiles into the output with TMA,
+// drops consumed ring lines from L2, frees the buffer, publishes finished tiles
+// on the segment counters).  Every wait is bounded
 // and records a flag in *err when it runs out.
 #pragma once
 #include "fourstep.cuh"
@@ -51,13 +52,15 @@ namespace fftseg {
 
 struct FourStepWlArgs {
     CUtensorMap tmA;     // input  [nseg][N1][N2], box [PW_A][256][1], swizzled
-    CUtensorMap tmB;     // ring   [slabs][N1/W_B][N2][W_B], box [PW_B][256][1][1], swizzled
+    CUtensorMap tmB;     // ring   [slabs][N1/PW_B][N2][PW_B], box [PW_B][256][1][1], swizzled
+    CUtensorMap tmR;     // ring, for the column tiles' stores: the same, box [PW_B][PW_A][N1/PW_B][1]
+                         // (ILV: ring [slabs][N1][N2][32], box [16][1][256][1])
     CUtensorMap tmO;     // output [nseg][N2][N1], box [PW_B][256][1], swizzled
-    float2 *ring;        // nr*cs segments, [slot*cs + sl][k1 / W_B][j2][k1 mod W_B]
+    float2 *ring;        // nr*cs segments, [slot*cs + sl][k1 / PW_B][j2][k1 mod PW_B]
     const float2 *twA;   // stage-2 twiddles of an N1-point line: [r-1][b] = w_{N1}^{b r}, r < P1, b < 32
     const float2 *twB;   // the same for N2
-    const float2 *w4t;   // per column tile ct, columns in pairs (c / 2, c mod 2 fastest):
-                         // [W_A/2][P1][2] w_n^{j2 j}, then [W_A/2][32][2] scale * w_n^{j2 P1 m}
+    const float2 *w4t;   // per column tile ct, columns by pair and half (WlPass::pair_of, c mod 2 fastest):
+                         // [W_A/2][P1][2] w_n^{j2 j}, then [32][W_A/2][2] scale * w_n^{j2 P1 m}
     int *ctr;            // [0] queue head, [1 + s] column tiles of s done, [1 + nc*cs + s] row tiles of s done
     int *err;
     int64_t nseg;
@@ -112,6 +115,13 @@ struct WlPass {
     // the XOR constant that applies the exchange permutation and the swizzle
     // to a row offset whose low three row bits are x
     __host__ __device__ static constexpr uint32_t K(int x) { return (uint32_t)(ROWB * x + 16 * ((x >> SWZ_S) & SWZ_M)); }
+    // The two lines that a half-warp holds (half h = 0, 1 of pair g): the even
+    // line 2 g and line 2 g ^ 5.  As with neighbouring lines one has the low
+    // and one the high 8 bytes of its 16-byte chunks, and bit 2 of the line
+    // number tells them apart too, which keeps the staged ring rows of the
+    // two (rows c of 128 bytes, swizzled by c mod 8) in different chunks.
+    // (Tiles of four lines have no bit 2: lines 2 g and 2 g + 1.)
+    __host__ __device__ static constexpr int line_of(int g, int h) { return h ? (2 * g) ^ (W >= 8 ? 5 : 1) : 2 * g; }
 };
 
 // ILV: the kernel's unit is 32 interleaved transforms (see FourStepWlArgs):
@@ -127,7 +137,7 @@ struct FourStepWlShape {
     static constexpr int64_t NS = ILV ? 32 * N : N;  // points of one unit (one ring slab)
     static constexpr int E = 1 << LOG_E;
     static constexpr int TC = E / 32;        // compute threads: 32 points each
-    static constexpr int TT = TC + 64;       // plus a loader warp and a retirer warp
+    static constexpr int TT = TC + 32 + 32 * NB;  // plus a loader warp and a retirer warp per buffer
     static constexpr int TSEG_A = ILV ? N2 : N2 / PA::W;  // column tiles per unit
     static constexpr int TSEG_B = ILV ? N1 : N1 / PB::W;  // row tiles per unit
     static_assert(!ILV || (PA::W == 32 && PB::W == 32), "interleaved units: tiles of 32 lines");
@@ -260,76 +270,62 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
 
     if (tid >= TC + 32) {
         // ============================================================= retirer
-        // Retires the CTA's tiles in buffer order as the compute warps finish
-        // them: frees a column tile's buffer at once (its ring stores came from
-        // registers); stores a row tile with TMA and frees its buffer once the
-        // store has read it; drops consumed ring lines from L2.  Segment
-        // counters are published in batches (one GPU-scope fence, then one add
-        // per tile) whenever no finished tile is waiting.  It waits only on this
-        // CTA's own warps and bulk stores.
-        const int lane = tid & 31;
+        // One warp per buffer: retires the tiles of its buffer as the compute
+        // warps finish them.  Stores a column tile into the ring and a row tile
+        // into the output with TMA, frees the buffer once the store has read
+        // it, drops a row tile's consumed ring lines from L2 and counts the
+        // tile on its segment's counter (a column tile once its ring stores
+        // have completed).  It waits only on this CTA's own warps and bulk
+        // stores.  (One retirer warp for all buffers, which could not free one
+        // while it waited for another's stores to complete, measured
+        // 1.98 ms at 65536 x 8192 against RETIRE_MS.)
+        const int lane = tid & 31, b = (tid - TC - 32) >> 5;
         const uint64_t stream_policy = policy_evict_first();  // the output is written once
-        int *const doneA = a.ctr + 1;
-        int *const doneB = a.ctr + 1 + (int64_t)a.nchunks * a.cs;
-        int *pend[4];
-        int npend = 0;
-        auto publish = [&]() {
-            if (lane == 0 && npend) {
-                fence_acq_rel_gpu();  // every write of the tiles (observed through `done`) first
-                for (int i = 0; i < 4; ++i)
-                    if (i < npend) atomicAdd(pend[i], 1);
-            }
-            npend = 0;
-        };
-        for (int64_t m = 0;; ++m) {
-            const int b = (int)(m % NB);
-            const uint32_t par = (uint32_t)(m / NB) & 1;
-            for (;;) {
-                const bool fin = __shfl_sync(0xffffffffu, (int)mbar_test_wait(&done[b], par), 0) != 0;
-                if (fin) break;
-                if (npend) {
-                    publish();
-                } else {
-                    mbar_wait(&done[b], par, a.err);
-                    break;
-                }
-            }
+        char *const src = reinterpret_cast<char *>(P + b * E);
+        for (uint32_t par = 0;; par ^= 1) {
+            mbar_wait(&done[b], par, a.err);
             const int kind = item[4 * b], s = item[4 * b + 1], w = item[4 * b + 2], slab = item[4 * b + 3];
+            __syncwarp();  // (the loader rewrites item[b] once the buffer is free)
             if (kind == KIND_END) break;
             if (kind == KIND_A || (kind == KIND_SKIP && w >= 0)) {
-                if (lane == 0) mbar_arrive(&empty[b]);
-                pend[npend++] = doneA + s;
-            } else {
-                const bool valid = kind == KIND_B;
-                const int rt = valid ? w : -w - 1;
                 if (lane == 0) {
-                    if (valid && a.out_power) {
-                        // one float box per 256 rows: [W_B floats][256 k2]
-                        constexpr int RBP = PB::W * 4;
+                    if (kind == KIND_A) {
+                        // (the ring lines' previous use, and their discard, by other
+                        // threads' generic accesses were observed by the loader)
+                        fence_proxy_async_global();
 #pragma unroll
-                        for (int q = 0; q < PB::NBOXY; ++q)
-                            tma_store_3d_hint(&a.tmO,
-                                              ILV ? rt * a.ilv_r + (s & ((1 << a.ilv_log_g) - 1)) * 32 : rt * PB::W,
-                                              q * 256, ILV ? s >> a.ilv_log_g : s,
-                                              reinterpret_cast<char *>(P + b * E) + q * 256 * RBP, stream_policy);
-                        bulk_commit();
-                        bulk_wait_read();  // the store has read the buffer
-                    } else if (valid) {
-#pragma unroll
-                        for (int p = 0; p < PB::NPANEL; ++p)
-#pragma unroll
-                            for (int q = 0; q < PB::NBOXY; ++q)
-                                tma_store_3d_hint(&a.tmO,
-                                                  (ILV ? rt * a.ilv_r + (s & ((1 << a.ilv_log_g) - 1)) * 32
-                                                       : rt * PB::W) + p * PB::PW,
-                                                  q * 256, ILV ? s >> a.ilv_log_g : s,
-                                                  reinterpret_cast<char *>(P + b * E) + p * PB::PANEL_BYTES +
-                                                      q * 256 * PB::ROWB,
-                                                  stream_policy);
+                        for (int p = 0; p < PA::NPANEL; ++p)
+                            if constexpr (ILV)  // rows k1 of 16 transforms, column j2 = w of the unit
+                                tma_store_4d(&a.tmR, p * PA::PW, w, 0, slab, src + p * PA::PANEL_BYTES);
+                            else  // [k1 / PW_B][column][k1 mod PW_B]
+                                tma_store_4d(&a.tmR, 0, w * PA::W + p * PA::PW, 0, slab, src + p * PA::PANEL_BYTES);
                         bulk_commit();
                         bulk_wait_read();  // the store has read the buffer
                     }
                     mbar_arrive(&empty[b]);
+                    bulk_wait_all();  // the ring stores have completed
+                    red_release_add(a.ctr + 1 + s, 1);
+                }
+            } else {
+                const bool valid = kind == KIND_B;
+                const int rt = valid ? w : -w - 1;
+                if (valid && lane == 0) {
+                    const int x = ILV ? rt * a.ilv_r + (s & ((1 << a.ilv_log_g) - 1)) * 32 : rt * PB::W;
+                    const int z = ILV ? s >> a.ilv_log_g : s;
+                    if (a.out_power) {
+                        // one float box per 256 rows: [W_B floats][256 k2]
+#pragma unroll
+                        for (int q = 0; q < PB::NBOXY; ++q)
+                            tma_store_3d_hint(&a.tmO, x, q * 256, z, src + q * 256 * PB::W * 4, stream_policy);
+                    } else {
+#pragma unroll
+                        for (int p = 0; p < PB::NPANEL; ++p)
+#pragma unroll
+                            for (int q = 0; q < PB::NBOXY; ++q)
+                                tma_store_3d_hint(&a.tmO, x + p * PB::PW, q * 256, z,
+                                                  src + p * PB::PANEL_BYTES + q * 256 * PB::ROWB, stream_policy);
+                    }
+                    bulk_commit();
                 }
                 if (valid) {
                     // the tile's ring block was consumed: drop its lines from L2
@@ -340,11 +336,13 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                         for (int l = lane; l < LINES; l += 32) discard_l2_line(tile + (int64_t)l * 16);
                     __syncwarp();
                 }
-                pend[npend++] = doneB + s;
+                if (lane == 0) {
+                    bulk_wait_read();  // the store has read the buffer
+                    mbar_arrive(&empty[b]);
+                    red_release_add(a.ctr + 1 + (int64_t)a.nchunks * a.cs + s, 1);
+                }
             }
-            if (npend == 4) publish();
         }
-        publish();
         if (lane == 0) bulk_wait_all();  // no store may outlive the CTA
         return;
     }
@@ -399,6 +397,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
         int t = 0;
         if (lane == 0) t = atomicAdd(a.ctr, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
+        int ends = 0;
         for (int64_t m = 0;; ++m) {
             const int b = (int)(m % NB);
             int isb = 0, c = 0, w = 0;
@@ -406,7 +405,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
             const bool end = t >= total;
             // the next tile is taken now: the atomic's latency overlaps this
             // tile's dependency probe, buffer wait and copies
-            int t_next = 0;
+            int t_next = t;
             if (lane == 0 && !end) t_next = atomicAdd(a.ctr, 1);
             if (lane == 0 && !end) {
                 decode(t, isb, c, w);
@@ -463,7 +462,8 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
 #pragma unroll
                                 for (int q = 0; q < PB::NBOXY; ++q)
                                     tma_load_4d(dst + p * PB::PANEL_BYTES + q * 256 * PB::ROWB, &a.tmB,
-                                                p * PB::PW, q * 256, tile, slab, &full[b]);
+                                                ILV ? p * PB::PW : 0, q * 256, ILV ? tile : tile * PB::NPANEL + p,
+                                                slab, &full[b]);
                         }
                     } else {
                         // an absent segment of the last chunk: nothing to load, but its
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                 }
             }
             t = __shfl_sync(0xffffffffu, t_next, 0);
-            if (end) break;
+            if (end && ++ends == NB) break;  // an end in every buffer
         }
         return;
     }
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
         const int u = tid % PA::GROUP;
         treg.load(TWA, (u & 7) | ((u >> 4) << 3));
     }
-    int bb = 0;
+    int bb = 0, ends = 0;
     uint32_t par = 0;
     char *const Pc = reinterpret_cast<char *>(P);
     for (;;) {
@@ -498,57 +498,80 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
         if (kind == KIND_END) {  // the retirer reads the end after this buffer's `done`
             __syncwarp();
             if ((tid & 31) == 0) mbar_arrive(&done[bb]);
-            break;
+            if (++ends == NB) break;
+            if (++bb == NB) {
+                bb = 0;
+                par ^= 1;
+            }
+            continue;
         }
         const uint32_t tb = (uint32_t)bb * Sh::TILE_BYTES;
         if (kind == KIND_A) {
             // column tile: lines are the columns j2 = W ct + c over j1
             using PS = PA;
-            const int s = item[4 * bb + 1], ct = item[4 * bb + 2], slab = item[4 * bb + 3];
+            const int ct = item[4 * bb + 2];
             const int group = tid / PS::GROUP, u = tid % PS::GROUP;
-            const int c = 2 * group + ((u >> 3) & 1), j = (u & 7) | ((u >> 4) << 3);
+            const int h = (u >> 3) & 1, c = PS::line_of(group, h), j = (u & 7) | ((u >> 4) << 3);
             float2 v[32];
             const float2 wcol = a.win_row ? __ldg(a.win_col + ct * PS::W + c) : float2{};
             wl_line<PS, S>(v, Pc, tb, c, j, group, TWA, TW_REG ? &treg : nullptr, a.win_row, wcol, a.err);
-            // times w_n^{j2 k1}, k1 = j + P m: w_n^{j2 j} w_n^{j2 P m} (scale folded in), into the ring
+            // times w_n^{j2 k1}, k1 = j + P m: w_n^{j2 j} w_n^{j2 P m} (scale folded in),
+            // staged in the tile's buffer for the retirer's TMA stores into the ring.
+            // (Storing the points to the ring from registers, 64-byte pieces at
+            // 2^16, took 2200 of a column tile's 5300 clocks; staged stores cost
+            // the compute warps one more pass over shared memory instead.)
             const float2 *Fb = F + bb * PS::FT;
-            const float2 f1 = Fb[((c >> 1) * PS::P + j) * 2 + (c & 1)];
-            const float2 *f2p = Fb + PS::W * PS::P + (c >> 1) * 64 + (c & 1);
-            // ring block layout [k1 / W_B][j2][k1 mod W_B], k1 = j + P m
-            // (ILV: [k1][j2][transform c of the unit])
-            constexpr int WB = PB::W;
-            constexpr int64_t BLK = (int64_t)Sh::N2 * WB;
-            const int j2 = ct * PS::W + c;
-            float2 *row = a.ring + (int64_t)slab * NS + (int64_t)j2 * WB;
-            float2 *dst = ILV ? a.ring + (int64_t)slab * NS + ct * WB + c + (int64_t)j * BLK
-                          : PS::P >= WB ? row + (int64_t)(j / WB) * BLK + (j % WB)
-                                        : row + j;
+            const float2 f1 = Fb[(group * PS::P + j) * 2 + h];
+            const float2 *f2p = Fb + PS::W * PS::P + group * 2 + h;
+            const int cc = c % PS::PW;  // column in its panel
+            const uint32_t pb = tb + (uint32_t)((c / PS::PW) * PS::PANEL_BYTES);
+            // ILV: rows k1 of the 32 transforms, in the line's own column.  Else
+            // panel by panel [k1 / PW_B][cc][k1 mod PW_B], rows of ROWB_B bytes
+            // with their TMA swizzle: other lines' slots, so every warp of the
+            // panel must have read its exchange rows first.
+            const uint32_t rb = pb + (uint32_t)(PS::ROWB * j) +
+                                (uint32_t)(16 * ((cc >> 1) ^ (((j & 7) >> PS::SWZ_S) & PS::SWZ_M)) + 8 * (cc & 1));
+            static_assert(PS::NPANEL <= 2, "named barriers 13 and 14");
+            if constexpr (ILV) wl_group_sync<PS::GROUP>(group);
+            else asm volatile("bar.sync %0, %1;" ::"r"(13 + c / PS::PW), "n"(TC / PS::NPANEL) : "memory");
+            // (factors in batches ahead of the stores: the compiler must keep a
+            // shared load behind an earlier shared store, and one load, product and
+            // store at a time cost 1980 clocks of latency per tile)
+            constexpr int NF = 8;
+            float2 f2[2][NF];
 #pragma unroll
-            for (int e = 0; e < PS::Q; ++e)
+            for (int i = 0; i < NF; ++i) f2[0][i] = f2p[i * PS::W];
 #pragma unroll
-                for (int r = 0; r < PS::P; ++r) {
-                    const int mm = e + PS::Q * r;
-                    const float2 f2 = f2p[2 * mm];
-                    const float2 wv = make_float2(f1.x * f2.x - f1.y * f2.y, f1.x * f2.y + f1.y * f2.x);
-                    // P >= W_B: k1 / W_B = j / W_B + m P / W_B, k1 mod W_B = j mod W_B;
-                    // else (W_B a multiple of P, j < P): k1 / W_B = m P / W_B, k1 mod W_B = j + m P mod W_B
-                    const int64_t off = ILV ? (int64_t)mm * PS::P * BLK
-                                        : PS::P >= WB ? (int64_t)mm * (PS::P / WB) * BLK
-                                                      : (int64_t)(mm * PS::P / WB) * BLK + (mm * PS::P) % WB;
-                    // (self-checking build: inside this segment's ring slab)
-                    if (FFTSEG_CHECK(dst + off - (a.ring + (int64_t)slab * NS) < NS &&
-                                         dst + off >= a.ring + (int64_t)slab * NS && slab < a.nr * a.cs,
-                                     a.err))
-                        dst[off] = twmul<S>(v[e * PS::P + r], wv);
+            for (int m0 = 0; m0 < 32; m0 += NF) {
+                if (m0 + NF < 32) {
+#pragma unroll
+                    for (int i = 0; i < NF; ++i) f2[(m0 / NF + 1) & 1][i] = f2p[(m0 + NF + i) * PS::W];
                 }
-            (void)s;
+#pragma unroll
+                for (int i = 0; i < NF; ++i) {
+                    const int mm = m0 + i, e = mm % PS::Q, r = mm / PS::Q;  // bin k1 = j + P mm
+                    const float2 w2 = f2[(m0 / NF) & 1][i];
+                    const float2 wv = make_float2(f1.x * w2.x - f1.y * w2.y, f1.x * w2.y + f1.y * w2.x);
+                    uint32_t off;
+                    if constexpr (ILV) {
+                        off = rb + PS::ROWB * PS::P * mm;
+                    } else {
+                        const int k1 = j + PS::P * mm, row = (k1 / PB::PW) * PS::PW + cc, x = k1 % PB::PW;
+                        off = pb + (uint32_t)(row * PB::ROWB) +
+                              (uint32_t)(16 * ((x >> 1) ^ ((row >> PB::SWZ_S) & PB::SWZ_M)) + 8 * (x & 1));
+                    }
+                    if (FFTSEG_CHECK(off - tb < Sh::TILE_BYTES, a.err))
+                        *reinterpret_cast<float2 *>(Pc + off) = twmul<S>(v[e * PS::P + r], wv);
+                }
+            }
+            fence_proxy_async();  // read by the retirer's TMA stores
         } else if (kind == KIND_B) {
             // row tile: lines are the rows k1 = W rt + c over j2; the bins
             // X[k1 + N1 k2] are staged as the output box [k2][k1 - W rt] in the
             // line's own column (the plan's scale is in the column pass's factors)
             using PS = PB;
             const int group = tid / PS::GROUP, u = tid % PS::GROUP;
-            const int c = 2 * group + ((u >> 3) & 1), j = (u & 7) | ((u >> 4) << 3);
+            const int c = PS::line_of(group, (u >> 3) & 1), j = (u & 7) | ((u >> 4) << 3);
             float2 v[32];
             if constexpr (TW_REG)
                 wl_line<PS, S>(v, Pc, tb, c, j, group, TWB, reinterpret_cast<const WlTw<PS> *>(&treg), nullptr,

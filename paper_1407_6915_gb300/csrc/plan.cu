@@ -247,10 +247,10 @@ int build_fourstep_wl(fftseg_plan p)
     if ((rc = stage2(&p->twA, n1))) return rc;
     if (l2 != l1 && (rc = stage2(&p->twB, n2))) return rc;
     {
-        // per column tile ct, its columns col (j2 = ct wa + col) in pairs, the
-        // pair's two columns side by side (so that the two lines a half-warp
-        // holds read adjacent entries): [wa/2][P1][2] w_n^{j2 j}, then
-        // [wa/2][32][2] scale * w_n^{j2 P1 m}
+        // per column tile ct, its columns col (j2 = ct wa + col) in the kernel's
+        // pairs (WlPass::line_of), the pair's two columns side by side (so that
+        // the two lines a half-warp holds read adjacent entries): [wa/2][P1][2]
+        // w_n^{j2 j}, then [32][wa/2][2] scale * w_n^{j2 P1 m}
         // (interleaved units: column tile j2 holds column j2 of 32 transforms,
         // so every column of tile j2 takes the factors of j2)
         const int64_t ft = wa * (p1 + 32);
@@ -260,12 +260,12 @@ int build_fourstep_wl(fftseg_plan p)
         for (int64_t tc = 0; tc < ntile * wa; ++tc) {
             const int64_t j2 = p->wl_ilv ? tc / wa : tc;
             float2 *t = h.data() + (tc / wa) * ft;
-            const int64_t col = tc % wa, pr = col >> 1, hc = col & 1;
+            const int64_t col = tc % wa, hc = col & 1, pr = (hc ? col ^ (wa >= 8 ? 5 : 1) : col) >> 1;
             host_roots(t1.data(), p1, p->n, j2);
             host_roots(t2.data(), 32, p->n, j2 * p1);
             for (int64_t j = 0; j < p1; ++j) t[(pr * p1 + j) * 2 + hc] = t1[(size_t)j];
             for (int m = 0; m < 32; ++m)
-                t[wa * p1 + (pr * 32 + m) * 2 + hc] = make_float2(t2[m].x * p->scale, t2[m].y * p->scale);
+                t[wa * p1 + m * wa + pr * 2 + hc] = make_float2(t2[m].x * p->scale, t2[m].y * p->scale);
         }
         if ((rc = upload(&p->w4t, h))) return rc;
     }
@@ -601,11 +601,13 @@ int exec_fourstep_wl(fftseg_plan p, const void *in, void *d_out, int64_t nseg, c
         rc = encode_tmap_3d_swz(&a.tmA, in, n2, n1, nseg, n2 * 8, n * 8, (uint32_t)pwa, 256, 8, (int)(pwa * 8));
     }
     if (rc == FFTSEG_OK) {
-        // ring blocks [slab][k1 / wb][j2][k1 mod wb]
-        const int64_t dims[4] = {wb, n2, n1 / wb, slabs};
-        const int64_t strides[3] = {wb * 8, n2 * wb * 8, n * 8};
+        // ring blocks [slab][k1 / pwb][j2][k1 mod pwb]
+        const int64_t dims[4] = {pwb, n2, n1 / pwb, slabs};
+        const int64_t strides[3] = {pwb * 8, n2 * pwb * 8, n * 8};
         const uint32_t box[4] = {(uint32_t)pwb, 256, 1, 1};
         rc = encode_tmap(&a.tmB, p->ring, 4, dims, strides, box, 8, (int)(pwb * 8));
+        const uint32_t rbox[4] = {(uint32_t)pwb, (uint32_t)pwa, (uint32_t)(n1 / pwb), 1};
+        if (rc == FFTSEG_OK) rc = encode_tmap(&a.tmR, p->ring, 4, dims, strides, rbox, 8, (int)(pwb * 8));
     }
     if (rc == FFTSEG_OK) {
         if (p->out_kind == FFTSEG_OUT_POWER)  // |X|^2: float rows of the row tile's wb lines
@@ -678,6 +680,8 @@ int exec_fourstep_ilv(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg
             const int64_t strides[3] = {32 * 8, n2 * 32 * 8, ns * 8};
             const uint32_t box[4] = {16, 256, 1, 1};
             rc = encode_tmap(&a.tmB, q->ring, 4, dims, strides, box, 8, 128);
+            const uint32_t rbox[4] = {16, 1, 256, 1};
+            if (rc == FFTSEG_OK) rc = encode_tmap(&a.tmR, q->ring, 4, dims, strides, rbox, 8, 128);
         }
         const bool power = p->out_kind == FFTSEG_OUT_POWER;
         if (rc == FFTSEG_OK) {  // X[t + R (k1 + N1 k2)] as [segment][k2][R k1 + t]
