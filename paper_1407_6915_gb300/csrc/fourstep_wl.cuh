@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
         // have completed).  It waits only on this CTA's own warps and bulk
         // stores.  (One retirer warp for all buffers, which could not free one
         // while it waited for another's stores to complete, measured
-        // 1.98 ms at 65536 x 8192 against RETIRE_MS.)
+        // 1.98 ms at 65536 x 8192 against 1.95.)
         const int lane = tid & 31, b = (tid - TC - 32) >> 5;
         const uint64_t stream_policy = policy_evict_first();  // the output is written once
         char *const src = reinterpret_cast<char *>(P + b * E);
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
     }
     if (tid >= TC) {
         // ============================================================== loader
-        // Takes tiles from the queue, in order, one ahead; probes a tile's
+        // Takes tiles from the queue, in order; probes a tile's
         // dependency, waits for a free buffer and issues the tile's TMA loads.
         const int lane = tid & 31;
         const int TA = a.cs * Sh::TSEG_A, TB = a.cs * Sh::TSEG_B;
@@ -394,8 +394,21 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
         // frames overlap: then the overlap is read again by the next frame
         const bool overlap = a.frame_rows > 0 && (int64_t)a.frame_rows * Sh::N2 < Sh::N;
         const uint64_t stream_policy = overlap ? policy_evict_unchanged() : policy_evict_first();
-        int t = 0;
-        if (lane == 0) t = atomicAdd(a.ctr, 1);
+        // Tickets are taken two tiles ahead and after a tile's copies are issued:
+        // the fence before the copies waits for every access of this thread in
+        // flight, so a ticket's round trip must not be among them (65536 x 8192:
+        // 1.85 ms with it in flight, 1.83 without).  With few
+        // tiles per CTA one is taken when it is needed, so that none sits behind
+        // another while a CTA idles.
+        const bool ahead = total >= 8 * (int)gridDim.x;
+        int t = 0, t1 = 0, t2 = 0;
+        if (lane == 0) {
+            t = atomicAdd(a.ctr, 1);
+            if (ahead) {
+                t1 = atomicAdd(a.ctr, 1);
+                t2 = atomicAdd(a.ctr, 1);
+            }
+        }
         t = __shfl_sync(0xffffffffu, t, 0);
         int ends = 0;
         for (int64_t m = 0;; ++m) {
@@ -403,10 +416,6 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
             int isb = 0, c = 0, w = 0;
             int64_t s = 0;
             const bool end = t >= total;
-            // the next tile is taken now: the atomic's latency overlaps this
-            // tile's dependency probe, buffer wait and copies
-            int t_next = t;
-            if (lane == 0 && !end) t_next = atomicAdd(a.ctr, 1);
             if (lane == 0 && !end) {
                 decode(t, isb, c, w);
                 s = (int64_t)c * a.cs + (isb ? w / Sh::TSEG_B : w / Sh::TSEG_A);
@@ -434,8 +443,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                     if (s < a.nseg) {
                         item[4 * b] = isb ? KIND_B : KIND_A;
                         item[4 * b + 2] = tile;
-                        if (isb) fence_proxy_async_global();  // ring data written by other CTAs' generic stores
-                        fence_proxy_async();
+                        if (isb) fence_proxy_async_global();  // ring data published through generic accesses
                         char *dst = reinterpret_cast<char *>(P + b * E);
                         if (!isb) {
                             mbar_expect_tx(&full[b], Sh::TILE_BYTES + Sh::F_BYTES);
@@ -474,7 +482,16 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                     }
                 }
             }
-            t = __shfl_sync(0xffffffffu, t_next, 0);
+            if (lane == 0 && !end) {
+                if (ahead) {
+                    t = t1;
+                    t1 = t2;
+                    t2 = atomicAdd(a.ctr, 1);
+                } else {
+                    t = atomicAdd(a.ctr, 1);
+                }
+            }
+            t = __shfl_sync(0xffffffffu, t, 0);
             if (end && ++ends == NB) break;  // an end in every buffer
         }
         return;
