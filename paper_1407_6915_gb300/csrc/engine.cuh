@@ -80,6 +80,18 @@ HDEV float2 csub(float2 a, float2 b)
 #endif
 }
 
+// a * s, s real
+HDEV float2 cscale(float2 a, float s)
+{
+#ifdef __CUDA_ARCH__
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(make_float2(s, s))));
+    return unpack2(r);
+#else
+    return make_float2(a.x * s, a.y * s);
+#endif
+}
+
 // a * s + b, s real
 HDEV float2 cfma(float2 a, float s, float2 b)
 {
@@ -99,6 +111,8 @@ HDEV float2 twmul(float2 a, float2 w)
     if (S < 0) return make_float2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
     return make_float2(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y);
 }
+
+HDEV float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
 // a * (sigma i)
 template <int S>
@@ -554,6 +568,15 @@ FDEV void tma_store_4d(const CUtensorMap *tmap, int x, int y, int z, int w, cons
                  : "memory");
 }
 
+// tma_store_3d for a 5-D map, at (x, y, z, w, v)
+FDEV void tma_store_5d(const CUtensorMap *tmap, int x, int y, int z, int w, int v, const void *src)
+{
+    asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4, %5}], [%6];" ::"l"(
+                     reinterpret_cast<uint64_t>(tmap)),
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(smem_u32(src))
+                 : "memory");
+}
+
 // wait until every committed bulk copy of this thread has completed its writes
 FDEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -652,6 +675,17 @@ FDEV void tma_load_3d_hint(void *dst, const CUtensorMap *tmap, int x, int y, int
         "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
         " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+
+// tma_load_4d with an L2 cache policy
+FDEV void tma_load_4d_hint(void *dst, const CUtensorMap *tmap, int x, int y, int z, int w, uint64_t *bar,
+                           uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar)), "l"(policy)
         : "memory");
 }
 

@@ -47,6 +47,7 @@
 // and records a flag in *err when it runs out.
 #pragma once
 #include "fourstep.cuh"
+#include "wl_tc.cuh"
 
 namespace fftseg {
 
@@ -55,6 +56,11 @@ struct FourStepWlArgs {
     CUtensorMap tmB;     // ring   [slabs][N1/PW_B][N2][PW_B], box [PW_B][256][1][1], swizzled
     CUtensorMap tmR;     // ring, for the column tiles' stores: the same, box [PW_B][PW_A][N1/PW_B][1]
                          // (ILV: ring [slabs][N1][N2][32], box [16][1][256][1])
+    // tensor-core lines (wl_tc.cuh): tmA as [nseg][b][r][16 columns], rows
+    // j1 = 16 r + b; the ring as [slabs][k1 / 16][b][r][16], rows j2 = 16 r + b
+    // as they are in shared memory, tmR box [16][1][16][16][1] without swizzle
+    // (row tiles are copied whole); w4t [2][16][WL_TC_FP] per column tile:
+    // w_n^{j2 k} [k][column], scale * w_n^{16 j2 q} [q][column]; twA: w_256^m
     CUtensorMap tmO;     // output [nseg][N2][N1], box [PW_B][256][1], swizzled
     float2 *ring;        // nr*cs segments, [slot*cs + sl][k1 / PW_B][j2][k1 mod PW_B]
     const float2 *twA;   // stage-2 twiddles of an N1-point line: [r-1][b] = w_{N1}^{b r}, r < P1, b < 32
@@ -124,11 +130,16 @@ struct WlPass {
     __host__ __device__ static constexpr int line_of(int g, int h) { return h ? (2 * g) ^ (W >= 8 ? 5 : 1) : 2 * g; }
 };
 
+// Columns of a row of the tensor-core lines' factor tables: the tile's 32 and
+// a pad that puts neighbouring rows in different banks.
+constexpr int WL_TC_FP = 36;
+
 // ILV: the kernel's unit is 32 interleaved transforms (see FourStepWlArgs):
 // a column tile is column j2 of all 32 of them and a row tile row k1 of all
 // 32, so that every tile's lines are the 32 transforms and its loads and
 // stores stay 256-byte runs.
-template <int LOG_N1, int LOG_N2, int LOG_E, int NB, int MINB, bool ILV = false>
+// PREC: FP32, or tensor-core lines (n = 256 x 256, no frames).
+template <int LOG_N1, int LOG_N2, int LOG_E, int NB, int MINB, bool ILV = false, int PREC = PREC_FP32>
 struct FourStepWlShape {
     using PA = WlPass<LOG_N1, LOG_E>;
     using PB = WlPass<LOG_N2, LOG_E>;
@@ -142,14 +153,17 @@ struct FourStepWlShape {
     static constexpr int TSEG_B = ILV ? N1 : N1 / PB::W;  // row tiles per unit
     static_assert(!ILV || (PA::W == 32 && PB::W == 32), "interleaved units: tiles of 32 lines");
     static constexpr uint32_t TILE_BYTES = E * sizeof(float2);
-    static constexpr uint32_t F_BYTES = PA::FT * sizeof(float2);
-    static constexpr int TWA = PA::TW, TWB = LOG_N1 == LOG_N2 ? 0 : PB::TW;
+    static constexpr bool TCL = PREC != PREC_FP32;
+    static_assert(!TCL || (LOG_N1 == 8 && LOG_N2 == 8 && LOG_E == 13 && !ILV), "tensor-core lines: 256 x 256");
+    static constexpr int FT = TCL ? 2 * 16 * WL_TC_FP : PA::FT;
+    static constexpr uint32_t F_BYTES = FT * sizeof(float2);
+    static constexpr int TWA = TCL ? 256 : PA::TW, TWB = LOG_N1 == LOG_N2 ? 0 : PB::TW;
     // P[NB] (1024-byte aligned) | F[NB] | stage-2 tables | full, done, empty [NB] | item [NB][4]
-    static constexpr size_t SMEM = (size_t)NB * E * sizeof(float2) + (size_t)NB * PA::FT * sizeof(float2) +
+    static constexpr size_t SMEM = (size_t)NB * E * sizeof(float2) + (size_t)NB * FT * sizeof(float2) +
                                    (size_t)(TWA + TWB) * sizeof(float2) + 3 * NB * sizeof(uint64_t) +
                                    NB * 4 * sizeof(int);
     static_assert(TC % 32 == 0 && TC >= 64, "whole compute warps");
-    static_assert((PA::FT * sizeof(float2)) % 16 == 0, "bulk copy of the factors");
+    static_assert((FT * sizeof(float2)) % 16 == 0, "bulk copy of the factors");
 };
 
 // Execution barrier over the 2P threads of a pair of lines.
@@ -231,19 +245,20 @@ FDEV void wl_line(float2 (&v)[32], char *Pc, uint32_t tb, int c, int j, int grou
     }
 }
 
-template <int LOG_N1, int LOG_N2, int LOG_E, int NB, int MINB, int S, bool ILV = false>
-__global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MINB, ILV>::TT, MINB)
+template <int LOG_N1, int LOG_N2, int LOG_E, int NB, int MINB, int S, bool ILV = false, int PREC = PREC_FP32>
+__global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MINB, ILV, PREC>::TT, MINB)
     k_fourstep_wl(const __grid_constant__ FourStepWlArgs a)
 {
-    using Sh = FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MINB, ILV>;
+    using Sh = FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MINB, ILV, PREC>;
     using PA = typename Sh::PA;
     using PB = typename Sh::PB;
-    constexpr int E = Sh::E, TC = Sh::TC, N1 = Sh::N1;
+    constexpr int E = Sh::E, TC = Sh::TC;
+    constexpr bool TCL = Sh::TCL;
     constexpr int64_t NS = Sh::NS;
     extern __shared__ __align__(1024) float2 sm[];
     float2 *const P = sm;
     float2 *const F = P + NB * E;
-    float2 *const TWA = F + NB * PA::FT;
+    float2 *const TWA = F + NB * Sh::FT;
     float2 *const TWB = LOG_N1 == LOG_N2 ? TWA : TWA + Sh::TWA;
     uint64_t *const full = reinterpret_cast<uint64_t *>(TWA + Sh::TWA + Sh::TWB);
     uint64_t *const done = full + NB;
@@ -295,7 +310,9 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                         fence_proxy_async_global();
 #pragma unroll
                         for (int p = 0; p < PA::NPANEL; ++p)
-                            if constexpr (ILV)  // rows k1 of 16 transforms, column j2 = w of the unit
+                            if constexpr (TCL)
+                                tma_store_5d(&a.tmR, 0, w * PA::NPANEL + p, 0, 0, slab, src + p * PA::PANEL_BYTES);
+                            else if constexpr (ILV)  // rows k1 of 16 transforms, column j2 = w of the unit
                                 tma_store_4d(&a.tmR, p * PA::PW, w, 0, slab, src + p * PA::PANEL_BYTES);
                             else  // [k1 / PW_B][column][k1 mod PW_B]
                                 tma_store_4d(&a.tmR, 0, w * PA::W + p * PA::PW, 0, slab, src + p * PA::PANEL_BYTES);
@@ -455,16 +472,21 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                                     // (ILV: column j2 = tile of the unit's 32 transforms, one
                                     // contiguous 256 x 32 block)
                                     const int x = (ILV ? 0 : tile * PA::W) + p * PA::PW;
-                                    if (a.frame_rows)  // rows of the signal from the frame's start
+                                    if constexpr (TCL)
+                                        tma_load_4d_hint(box, &a.tmA, x, 0, 0, (int)s, &full[b], stream_policy);
+                                    else if (a.frame_rows)  // rows of the signal from the frame's start
                                         tma_load_2d_hint(box, &a.tmA, x, (int)s * a.frame_rows + q * 256, &full[b],
                                                          stream_policy);
                                     else
                                         tma_load_3d_hint(box, &a.tmA, x, q * 256, ILV ? (int)s * Sh::N2 + tile : (int)s,
                                                          &full[b], stream_policy);
                                 }
-                            tma_load_1d(F + b * PA::FT, a.w4t + (int64_t)tile * PA::FT, Sh::F_BYTES, &full[b]);
+                            tma_load_1d(F + b * Sh::FT, a.w4t + (int64_t)tile * Sh::FT, Sh::F_BYTES, &full[b]);
                         } else {
                             mbar_expect_tx(&full[b], Sh::TILE_BYTES);
+                            if constexpr (TCL)
+                                tma_load_1d(dst, a.ring + (int64_t)slab * NS + (int64_t)tile * E, Sh::TILE_BYTES, &full[b]);
+                            else
 #pragma unroll
                             for (int p = 0; p < PB::NPANEL; ++p)
 #pragma unroll
@@ -500,8 +522,20 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
     // ================================================================ compute
     // with one line length for both passes a lane keeps the same j, so its
     // stage-2 twiddles live in registers for the whole launch
-    constexpr bool TW_REG = LOG_N1 == LOG_N2;
-    WlTw<PA> treg;
+    constexpr bool TW_REG = LOG_N1 == LOG_N2 && !TCL;
+    [[maybe_unused]] WlTw<PA> treg;
+    // tensor-core lines: the DFT matrix and the lane's twiddles w_256^{b k},
+    // b = 2 G + (t >> 1), k = g + 8 mt, for the whole launch
+    [[maybe_unused]] WlTcF tcf;
+    [[maybe_unused]] float2 tctw[8][2];
+    [[maybe_unused]] const int tg = (tid & 31) >> 2, tt = tid & 3, tp = tid >> 7, tw = (tid >> 5) & 3;
+    if constexpr (TCL) {
+        tcf.init<S, PREC>(tg, tt);
+#pragma unroll
+        for (int G = 0; G < 8; ++G)
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) tctw[G][mt] = TWA[(2 * G + (tt >> 1)) * (tg + 8 * mt)];
+    }
     if constexpr (TW_REG) {
         const int u = tid % PA::GROUP;
         treg.load(TWA, (u & 7) | ((u >> 4) << 3));
@@ -523,7 +557,76 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
             continue;
         }
         const uint32_t tb = (uint32_t)bb * Sh::TILE_BYTES;
-        if (kind == KIND_A) {
+        if constexpr (TCL) {
+            if (kind == KIND_A || kind == KIND_B) {
+                float d[8][2][4];
+                const uint32_t pb = tb + (uint32_t)(tp * PA::PANEL_BYTES);
+                const int tile = item[4 * bb + 2];
+                if (kind == KIND_A) wl_tc_line<S, PREC, false>(d, Pc, pb, tw, tg, tt, 0, tcf, tctw);
+                else wl_tc_line<S, PREC, true>(d, Pc, pb, tw, tg, tt, (2 * tile + tp) & 3, tcf, tctw);
+                const int c0 = 2 * tw + 8 * (tt & 1);  // the lane's first line in its panel
+                if (kind == KIND_A) {
+                    // times w_n^{j2 k1} (two factors, scale folded in), staged as [q][column][16 k]
+                    const float4 *F1 = reinterpret_cast<const float4 *>(F + bb * Sh::FT + 16 * tp + c0) +
+                                       (tt >> 1) * (WL_TC_FP / 2);
+                    const float4 *F2 = reinterpret_cast<const float4 *>(F + bb * Sh::FT + 16 * WL_TC_FP + 16 * tp + c0) +
+                                       tg * (WL_TC_FP / 2);
+                    float4 f1[8], f2[2];
+#pragma unroll
+                    for (int G = 0; G < 8; ++G) f1[G] = F1[G * WL_TC_FP];
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt) f2[mt] = F2[mt * 4 * WL_TC_FP];
+                    // every warp of the panel has read its exchange rows
+                    asm volatile("bar.sync %0, %1;" ::"r"(13 + tp), "n"(TC / PA::NPANEL) : "memory");
+                    const uint32_t x = (uint32_t)((tg & 3) ^ (4 * (tt & 1)) ^ ((2 * tile + tp) & 7));
+                    const uint32_t sb = pb + 2048 * tg + 128 * c0 + 16 * x + 8 * (tt >> 1);
+#pragma unroll
+                    for (int G = 0; G < 8; ++G)
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt) {
+                            const float2 w0 = cmul(make_float2(f1[G].x, f1[G].y), make_float2(f2[mt].x, f2[mt].y));
+                            const float2 w1 = cmul(make_float2(f1[G].z, f1[G].w), make_float2(f2[mt].z, f2[mt].w));
+                            const uint32_t off = (sb ^ (16u * G)) + 16384u * mt;
+                            if (FFTSEG_CHECK(off + 128 - tb < Sh::TILE_BYTES, a.err)) {
+                                *reinterpret_cast<float2 *>(Pc + off) =
+                                    twmul<S>(make_float2(d[G][mt][0], d[G][mt][2]), w0);
+                                *reinterpret_cast<float2 *>(Pc + off + 128) =
+                                    twmul<S>(make_float2(d[G][mt][1], d[G][mt][3]), w1);
+                            }
+                        }
+                } else if (a.out_power) {
+                    // |X|^2 as float rows [k2][32 lines], like the FP32 lines'
+                    asm volatile("bar.sync 15, %0;" ::"n"(TC) : "memory");
+                    const int c = 16 * tp + c0;
+#pragma unroll
+                    for (int G = 0; G < 8; ++G)
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt) {
+                            const int k2 = 2 * G + (tt >> 1) + 16 * (tg + 8 * mt);
+                            const uint32_t off = tb + (uint32_t)(k2 * 128 + (((c >> 2) ^ (k2 & 7)) << 4) + (c & 3) * 4);
+                            if (FFTSEG_CHECK(off - tb < Sh::TILE_BYTES, a.err))
+                                *reinterpret_cast<float2 *>(Pc + off) =
+                                    make_float2(power_of(make_float2(d[G][mt][0], d[G][mt][2])),
+                                                power_of(make_float2(d[G][mt][1], d[G][mt][3])));
+                        }
+                } else {
+                    // the output box [k2][16 lines] with its TMA swizzle
+                    asm volatile("bar.sync %0, %1;" ::"r"(13 + tp), "n"(TC / PB::NPANEL) : "memory");
+                    const uint32_t lo = (uint32_t)(tt >> 1);
+                    const uint32_t ob = pb + 2048 * tg + 128 * lo + 16 * ((uint32_t)(c0 >> 1) ^ lo);
+#pragma unroll
+                    for (int G = 0; G < 8; ++G)
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt) {
+                            const uint32_t off = (ob ^ (256u * G + 16u * ((2 * G) & 7))) + 16384u * mt;
+                            if (FFTSEG_CHECK(off - tb < Sh::TILE_BYTES, a.err))
+                                *reinterpret_cast<float4 *>(Pc + off) =
+                                    make_float4(d[G][mt][0], d[G][mt][2], d[G][mt][1], d[G][mt][3]);
+                        }
+                }
+                fence_proxy_async();  // read by the retirer's TMA stores
+            }
+        } else if (kind == KIND_A) {
             // column tile: lines are the columns j2 = W ct + c over j1
             using PS = PA;
             const int ct = item[4 * bb + 2];
@@ -537,7 +640,7 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
             // (Storing the points to the ring from registers, 64-byte pieces at
             // 2^16, took 2200 of a column tile's 5300 clocks; staged stores cost
             // the compute warps one more pass over shared memory instead.)
-            const float2 *Fb = F + bb * PS::FT;
+            const float2 *Fb = F + bb * Sh::FT;
             const float2 f1 = Fb[(group * PS::P + j) * 2 + h];
             const float2 *f2p = Fb + PS::W * PS::P + group * 2 + h;
             const int cc = c % PS::PW;  // column in its panel

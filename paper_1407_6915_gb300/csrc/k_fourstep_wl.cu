@@ -14,11 +14,11 @@ namespace {
 // 4-27 % slower at 2^17..2^20.)
 constexpr int kWlLogE = 13, kWlNb = 3, kWlMinB = 1;
 
-template <int LOG_N1, int LOG_N2, int S, bool ILV = false>
+template <int LOG_N1, int LOG_N2, int S, bool ILV = false, int PREC = PREC_FP32>
 cudaError_t wl_t(const FourStepWlArgs &a, cudaStream_t st)
 {
-    using Sh = FourStepWlShape<LOG_N1, LOG_N2, kWlLogE, kWlNb, kWlMinB, ILV>;
-    auto k = k_fourstep_wl<LOG_N1, LOG_N2, kWlLogE, kWlNb, kWlMinB, S, ILV>;
+    using Sh = FourStepWlShape<LOG_N1, LOG_N2, kWlLogE, kWlNb, kWlMinB, ILV, PREC>;
+    auto k = k_fourstep_wl<LOG_N1, LOG_N2, kWlLogE, kWlNb, kWlMinB, S, ILV, PREC>;
     // per device: the occupancy of this instantiation (the grid is the
     // resident CTAs of the GPU the launch goes to)
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
@@ -62,8 +62,14 @@ cudaError_t launch_fourstep_wl_ilv(int sign, const FourStepWlArgs &a, cudaStream
     return sign < 0 ? wl_t<8, 8, -1, true>(a, st) : wl_t<8, 8, 1, true>(a, st);
 }
 
-cudaError_t launch_fourstep_wl(int log_n, int sign, const FourStepWlArgs &a, cudaStream_t st)
+cudaError_t launch_fourstep_wl(int log_n, int sign, int prec, const FourStepWlArgs &a, cudaStream_t st)
 {
+    if (prec != PREC_FP32) {
+        if (log_n != 16) return cudaErrorInvalidValue;
+        if (prec == PREC_FP16)
+            return sign < 0 ? wl_t<8, 8, -1, false, PREC_FP16>(a, st) : wl_t<8, 8, 1, false, PREC_FP16>(a, st);
+        return sign < 0 ? wl_t<8, 8, -1, false, PREC_BF16>(a, st) : wl_t<8, 8, 1, false, PREC_BF16>(a, st);
+    }
     switch (log_n) {
         case 16: return wl_s<8, 8>(sign, a, st);
         case 17: return wl_s<9, 8>(sign, a, st);

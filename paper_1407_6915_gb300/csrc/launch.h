@@ -75,9 +75,10 @@ struct FourStepHwArgs;
 cudaError_t launch_fourstep_hw(int sign, const FourStepHwArgs &a, cudaStream_t st);
 // Lane-line persistent four-step kernel for n = 2^16..2^20 (FP32, complex
 // output): lines of 256..1024 points with 32 points per lane, a queue of
-// column and row tiles, loader and retirer warps, swizzled TMA tiles.
+// column and row tiles, loader and retirer warps, swizzled TMA tiles.  prec as
+// for launch_block (tensor-core lines at n = 2^16).
 struct FourStepWlArgs;
-cudaError_t launch_fourstep_wl(int log_n, int sign, const FourStepWlArgs &a, cudaStream_t st);
+cudaError_t launch_fourstep_wl(int log_n, int sign, int prec, const FourStepWlArgs &a, cudaStream_t st);
 // The same kernel at n = 2^16 over interleaved units of 32 transforms
 // (a.ilv_r transforms per segment, a.nseg units).
 cudaError_t launch_fourstep_wl_ilv(int sign, const FourStepWlArgs &a, cudaStream_t st);

@@ -30,19 +30,28 @@ constexpr int kRingNr = 3;
 
 bool is_pow2(int64_t n) { return n >= 1 && (n & (n - 1)) == 0; }
 
-// FP32 complex output on the persistent four-step path, not asked for the
-// producer or CTA-tile kernels: the lane-local-line kernels can run it.
+// FP32 on the persistent four-step path, not asked for the producer or
+// CTA-tile kernels: the lane-local-line kernels can run it.
 bool lane_kernels_apply(const fftseg_plan_s *p)
 {
     return p->precision == FFTSEG_PREC_FP32 &&
+           !(p->flags & (FFTSEG_FLAG_FOURSTEP_PRODUCER | FFTSEG_FLAG_FOURSTEP_TILES));
+}
+// Tensor-core precisions at n = 256 x 256: the lane-line kernel with
+// tensor-core lines (wl_tc.cuh) instead of the CTA-tile kernel, whose operands
+// and results all pass through shared memory (1024 segments: 1159 us against
+// 455 us).  Longer ones have lines that are not 16 x 16 points.
+bool uses_wl_tc(const fftseg_plan_s *p)
+{
+    return p->precision != FFTSEG_PREC_FP32 && p->log_n == 16 &&
            !(p->flags & (FFTSEG_FLAG_FOURSTEP_PRODUCER | FFTSEG_FLAG_FOURSTEP_TILES));
 }
 // n = 2^16..2^20: the lane-line kernel (fourstep_wl.cuh), measured faster
 // than the warp-line kernel at 2^16 (0.60 against 0.59 of the copy peak).
 bool uses_fourstep_wl(const fftseg_plan_s *p)
 {
-    return lane_kernels_apply(p) && p->log_n >= 16 && p->log_n <= 20 &&
-           !(p->flags & FFTSEG_FLAG_FOURSTEP_WARP_LINES);
+    return uses_wl_tc(p) || (lane_kernels_apply(p) && p->log_n >= 16 && p->log_n <= 20 &&
+                             !(p->flags & FFTSEG_FLAG_FOURSTEP_WARP_LINES));
 }
 // n = 2^21..2^24: the outer radix-R pass and the lane-line kernel over
 // interleaved transforms of 2^16 points (two HBM passes).
@@ -232,7 +241,7 @@ int build_fourstep_wl(fftseg_plan p)
     p->log_n1 = l1;
     p->log_n2 = l2;
     const int64_t n1 = int64_t(1) << l1, n2 = int64_t(1) << l2;
-    const int64_t p1 = n1 / 32, p2 = n2 / 32;
+    const int64_t p1 = n1 / 32;
     const int64_t wa = (int64_t(1) << le) / n1;  // columns per column tile
     p->log_wa = le - l1;
     p->log_wb = le - l2;
@@ -244,9 +253,28 @@ int build_fourstep_wl(fftseg_plan p)
         for (int64_t r = 1; r < P; ++r) host_roots(h.data() + (r - 1) * 32, 32, L, r);
         return upload(dst, h);
     };
-    if ((rc = stage2(&p->twA, n1))) return rc;
+    const bool tc = p->precision != FFTSEG_PREC_FP32;
+    if (tc) {
+        // tensor-core lines: w_256^m, and per column tile of 32 columns
+        // w_n^{j2 k} [k][column] then scale * w_n^{16 j2 q} [q][column], k, q < 16,
+        // rows of WL_TC_FP columns
+        std::vector<float2> r(256), h((size_t)(n2 / wa * 32 * WL_TC_FP)), t(16);
+        host_roots(r.data(), 256, 256, 1);
+        if ((rc = upload(&p->twA, r))) return rc;
+        for (int64_t j2 = 0; j2 < n2; ++j2) {
+            float2 *f = h.data() + (j2 / wa) * 32 * WL_TC_FP + j2 % wa;
+            host_roots(t.data(), 16, p->n, j2);
+            for (int k = 0; k < 16; ++k) f[k * WL_TC_FP] = t[(size_t)k];
+            host_roots(t.data(), 16, p->n, j2 * 16);
+            for (int q = 0; q < 16; ++q)
+                f[(16 + q) * WL_TC_FP] = make_float2(t[(size_t)q].x * p->scale, t[(size_t)q].y * p->scale);
+        }
+        if ((rc = upload(&p->w4t, h))) return rc;
+    } else if ((rc = stage2(&p->twA, n1))) {
+        return rc;
+    }
     if (l2 != l1 && (rc = stage2(&p->twB, n2))) return rc;
-    {
+    if (!tc) {
         // per column tile ct, its columns col (j2 = ct wa + col) in the kernel's
         // pairs (WlPass::line_of), the pair's two columns side by side (so that
         // the two lines a half-warp holds read adjacent entries): [wa/2][P1][2]
@@ -600,7 +628,15 @@ int exec_fourstep_wl(fftseg_plan p, const void *in, void *d_out, int64_t nseg, c
     } else {
         rc = encode_tmap_3d_swz(&a.tmA, in, n2, n1, nseg, n2 * 8, n * 8, (uint32_t)pwa, 256, 8, (int)(pwa * 8));
     }
-    if (rc == FFTSEG_OK) {
+    if (uses_wl_tc(p)) {
+        // rows j1 = 16 r + b in the order [b][r]; the ring rows j2 likewise, as they are in shared memory
+        const int64_t dims[4] = {n2, 16, 16, nseg}, strides[3] = {16 * n2 * 8, n2 * 8, n * 8};
+        const uint32_t box[4] = {16, 16, 16, 1};
+        rc = encode_tmap(&a.tmA, in, 4, dims, strides, box, 8, 128);
+        const int64_t rdims[5] = {16, 16, 16, 16, slabs}, rstrides[4] = {128, 16 * 128, 256 * 128, n * 8};
+        const uint32_t rbox[5] = {16, 1, 16, 16, 1};
+        if (rc == FFTSEG_OK) rc = encode_tmap(&a.tmR, p->ring, 5, rdims, rstrides, rbox, 8, 0);
+    } else if (rc == FFTSEG_OK) {
         // ring blocks [slab][k1 / pwb][j2][k1 mod pwb]
         const int64_t dims[4] = {pwb, n2, n1 / pwb, slabs};
         const int64_t strides[3] = {pwb * 8, n2 * pwb * 8, n * 8};
@@ -634,7 +670,7 @@ int exec_fourstep_wl(fftseg_plan p, const void *in, void *d_out, int64_t nseg, c
     a.stall = (p->flags & FFTSEG_FLAG_TEST_STALL) ? 1 : 0;
     cudaError_t e = cudaMemsetAsync(p->ctr, 0, (size_t)(1 + 2 * nc * cs) * sizeof(int), st);
     if (e != cudaSuccess) return cuda_error(e, "four-step counter reset");
-    e = launch_fourstep_wl(p->log_n, p->direction, a, st);
+    e = launch_fourstep_wl(p->log_n, p->direction, kernel_prec(p), a, st);
     if (e != cudaSuccess) return cuda_error(e, "four-step kernel launch");
     count_launches(1);
     return FFTSEG_OK;

@@ -40,15 +40,15 @@ FDEV uint32_t pack_hi(float a, float b, float &ra, float &rb)
     uint32_t u;
     if (PREC == PREC_FP16) {
         const __half2 h = __floats2half2_rn(a, b);
-        const float2 f = __half22float2(h);
-        ra = a - f.x;
-        rb = b - f.y;
+        const float2 r = csub(make_float2(a, b), __half22float2(h));
+        ra = r.x;
+        rb = r.y;
         u = *reinterpret_cast<const uint32_t *>(&h);
     } else {
         const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-        const float2 f = __bfloat1622float2(h);
-        ra = a - f.x;
-        rb = b - f.y;
+        const float2 r = csub(make_float2(a, b), __bfloat1622float2(h));
+        ra = r.x;
+        rb = r.y;
         u = *reinterpret_cast<const uint32_t *>(&h);
     }
     return u;

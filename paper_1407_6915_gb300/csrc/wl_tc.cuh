@@ -1,0 +1,157 @@
+// Tensor-core lines of the lane-line four-step kernel at 256 x 256: both
+// radix-16 stages of a 256-point line as 32 x 32 real products on
+// mma.sync.m16n8k16 with split hi+lo 16-bit operands (tc.cuh has the method:
+// Y ~ Fh Xl + Fl Xh + Fh Xh, FP32 accumulation).
+//
+// The DFT matrix is the A operand and eight butterflies are the columns of B,
+// so that the fragments are what a lane can read and write directly, with no
+// staging of operands: with g = lane / 4, t = lane % 4
+//   B: lane (g, t) holds points t + 4 i, i < 4, of butterfly g (re and im are
+//      neighbouring k indices), four 8-byte loads from the tile;
+//   C: lane (g, t) holds bins g and g + 8 (rows g and g + 8 of a 16-row tile
+//      are the re and im of one bin) of butterflies 2 t and 2 t + 1.
+// A warp holds four lines of a panel, columns 2 w + {0, 1, 8, 9} (w: the warp's
+// number in its panel), and runs them in eight groups of eight butterflies:
+// butterfly g of group G is line 2 w + (g & 1) + 8 ((g >> 1) & 1), butterfly
+// b = 2 G + (g >> 2).  So C's two butterflies are one b of two neighbouring
+// lines: a 16-byte store.
+//
+// FP16 operands are scaled into range by a power of two taken from the group's
+// largest component (one warp reduction per group, scaled back exactly).
+// Elements within 2^-15 of that maximum keep all 22 bits of the split; for
+// smaller ones the error stays below 2^-38 of the maximum.
+//
+// Tile rows: element (hi, lo) of a line, hi, lo < 16, is in row 16 hi + lo, its
+// 16-byte chunk at (column / 2) ^ (lo & 7) ^ X(hi).  Input tiles hold point
+// 16 lo + hi there (butterfly hi, point lo of its sixteen), which the tensor
+// map of the input and the ring's row order provide.  Column tiles: X = 0, the
+// TMA swizzle.  Row tiles: X(hi) = 4 (hi >> 3) ^ (q & 3), q = k1 / 16, the
+// pattern that lets the column pass write its staged ring rows without bank
+// conflicts; the ring holds the rows as they are in shared memory.  The
+// exchange puts bin k of butterfly b at (k, b ^ 2 (k & 1)).  Every access is
+// conflict-free but the row tiles' staged output (two-way).
+//
+// 1024 segments of 65536 points, FP16 hi+lo: 455 us (BF16: 390 us) against
+// 1159 us on the CTA-tile kernel, whose operands, hi and lo, and results all
+// pass through shared memory once more per stage.  Tensor pipe 37 % active,
+// shared-memory pipe 35 %, issue 35 %: bound by latency, with two compute warps
+// per scheduler.
+#pragma once
+#include "tc.cuh"
+
+namespace fftseg {
+
+// The DFT matrix as A fragments: [row tile][k step][a0..a3], hi and lo.
+struct WlTcF {
+    uint32_t h[2][2][4], l[2][2][4];
+    template <int S, int PREC>
+    FDEV void init(int g, int t)
+    {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int kt = 0; kt < 2; ++kt)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int m = g + 8 * mt, r = t + 4 * (2 * kt + q);
+                    double sd, cd;
+                    sincospi((double)((r * m) & 15) / 8.0, &sd, &cd);
+                    const float c = (float)cd, s = (float)(S * sd);
+                    float la, lb;
+                    h[mt][kt][2 * q] = pack_hi<PREC>(c, -s, la, lb);  // row re(m)
+                    l[mt][kt][2 * q] = pack_lo<PREC>(la, lb);
+                    h[mt][kt][2 * q + 1] = pack_hi<PREC>(s, c, la, lb);  // row im(m)
+                    l[mt][kt][2 * q + 1] = pack_lo<PREC>(la, lb);
+                }
+    }
+};
+
+// Eight butterflies: d[mt] = (re, re', im, im') of bin g + 8 mt of butterflies
+// 2 t and 2 t + 1 from this lane's points x[i] = t + 4 i of butterfly g.
+template <int PREC>
+FDEV void wl_tc_group(float (&d)[2][4], const float2 (&x)[4], const WlTcF &F)
+{
+    float sc = 1.f, inv = 1.f;
+    if constexpr (PREC == PREC_FP16) {
+        float mx = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mx = fmaxf(mx, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
+        const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+        int e = (int)(top >> 23) - 127;  // floor(log2) of a normal maximum
+        e = e < -100 ? -100 : (e > 100 ? 100 : e);
+        sc = __uint_as_float((uint32_t)(127 + 13 - e) << 23);
+        inv = __uint_as_float((uint32_t)(127 - 13 + e) << 23);
+    }
+    uint32_t xh[4], xl[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float la, lb;
+        const float2 y = PREC == PREC_FP16 ? cscale(x[i], sc) : x[i];
+        xh[i] = pack_hi<PREC>(y.x, y.y, la, lb);
+        xl[i] = pack_lo<PREC>(la, lb);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) d[i >> 2][i & 3] = 0.f;
+    // (products in an order that alternates between accumulators, or between
+    // those of two groups, measured the same)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+        for (int kt = 0; kt < 2; ++kt) {
+            mma16816<PREC>(d[mt], F.h[mt][kt], xl[2 * kt], xl[2 * kt + 1]);
+            mma16816<PREC>(d[mt], F.l[mt][kt], xh[2 * kt], xh[2 * kt + 1]);
+            mma16816<PREC>(d[mt], F.h[mt][kt], xh[2 * kt], xh[2 * kt + 1]);
+        }
+        if constexpr (PREC == PREC_FP16) {
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+                const float2 y = cscale(make_float2(d[mt][i], d[mt][i + 1]), inv);
+                d[mt][i] = y.x;
+                d[mt][i + 1] = y.y;
+            }
+        }
+    }
+}
+
+// This warp's four lines of the panel at byte offset pb, in place in the tile
+// buffer; ROWS: a row tile whose panel is q = qx mod 4.  On return d[G][mt]
+// holds (re, re', im, im') of bin k + 16 (g + 8 mt), k = 2 G + (t >> 1), of
+// lines 2 w + 8 (t & 1) and the next.
+template <int S, int PREC, bool ROWS>
+FDEV void wl_tc_line(float (&d)[8][2][4], char *Pc, uint32_t pb, int w, int g, int t, int qx, const WlTcF &F,
+                     const float2 (&tw)[8][2])
+{
+    auto KX = [](uint32_t x) { return 128 * x + 16 * (x & 7); };  // row and chunk bits of lo
+    const uint32_t X = ROWS ? (uint32_t)qx : 0u;
+    const uint32_t lc = (uint32_t)(w + 4 * ((g >> 1) & 1)) ^ X, rd = pb + 2048 * (g >> 2) + 8 * (g & 1);
+    const uint32_t lw = (uint32_t)(w + 4 * (t & 1)) ^ X;
+    auto pass = [&](uint32_t t0) {
+        const uint32_t base = rd + 128 * t0 + 16 * (lc ^ t0);
+#pragma unroll
+        for (int G = 0; G < 8; ++G) {
+            float2 x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                x[i] = *reinterpret_cast<const float2 *>(Pc + ((base ^ KX(4 * i) ^ (ROWS && G >= 4 ? 64u : 0u)) +
+                                                               4096u * G));
+            wl_tc_group<PREC>(d[G], x, F);
+        }
+    };
+    pass((uint32_t)t);
+    __syncwarp();  // every lane has read its points
+    const uint32_t lo = (uint32_t)((t >> 1) ^ (2 * (g & 1)));
+    const uint32_t wb = pb + 2048 * g + 128 * lo + 16 * (lw ^ lo);
+#pragma unroll
+    for (int G = 0; G < 8; ++G)
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            const float2 a = twmul<S>(make_float2(d[G][mt][0], d[G][mt][2]), tw[G][mt]);
+            const float2 b = twmul<S>(make_float2(d[G][mt][1], d[G][mt][3]), tw[G][mt]);
+            *reinterpret_cast<float4 *>(Pc + ((wb ^ KX(2 * G) ^ (ROWS && mt ? 64u : 0u)) + 16384u * mt)) =
+                make_float4(a.x, a.y, b.x, b.y);
+        }
+    __syncwarp();
+    pass((uint32_t)(t ^ (2 * (g >> 2))));
+}
+
+}  // namespace fftseg
