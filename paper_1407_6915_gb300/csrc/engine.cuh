@@ -386,10 +386,93 @@ HDEV void dft_odd(float2 *v)
     v[0] = X0;
 }
 
+// cos and sin(2 pi m / R) at compile time, by their Taylor series on
+// [0, pi/4] (18 terms of the angle's powers; the argument's octant and the
+// symmetries give the rest), rounded once to float.
+__host__ __device__ constexpr double ct_series(double x, bool sine)
+{
+    double term = sine ? x : 1.0, sum = term;
+    for (int i = sine ? 2 : 1; i < 18; i += 2) {
+        term *= -x * x / ((double)i * (i + 1));
+        sum += term;
+    }
+    return sum;
+}
+__host__ __device__ constexpr double ct_cos(int m, int R)
+{
+    m = ((m % R) + R) % R;
+    if (2 * m > R) m = R - m;              // cos(2 pi - a) = cos(a)
+    if (4 * m > R) return -ct_cos(R - 2 * m, 2 * R);  // cos(pi - a) = -cos(a)
+    const double a = 6.283185307179586476925286766559 * m / R;
+    if (8 * m <= R) return ct_series(a, false);
+    return ct_series(1.5707963267948966192313216916398 - a, true);  // cos(a) = sin(pi/2 - a)
+}
+__host__ __device__ constexpr double ct_sin(int m, int R) { return ct_cos(4 * m - R, 4 * R); }  // sin(a) = cos(a - pi/2)
+
+// a * w_R^M, w_R = exp(sigma 2 pi i / R)
+template <int M, int R, int S>
+HDEV float2 rot_const(float2 a)
+{
+    if constexpr (M % R == 0) return a;
+    else if constexpr (4 * M == R) return mul_si<S>(a);
+    else if constexpr (2 * M == R) return make_float2(-a.x, -a.y);
+    else {
+        constexpr float c = (float)ct_cos(M, R), s = (float)(S * ct_sin(M, R));
+        return make_float2(a.x * c - a.y * s, a.y * c + a.x * s);
+    }
+}
+
+// Composite radix R = A B with j = B j1 + j2, k = k1 + A k2, as dft16.
+template <int A, int B, int S, int J2 = 1, int K1 = 1>
+HDEV void dft_ab_twiddle(float2 *v)
+{
+    if constexpr (J2 < B) {
+        v[K1 * B + J2] = rot_const<J2 * K1, A * B, S>(v[K1 * B + J2]);
+        if constexpr (K1 + 1 < A) dft_ab_twiddle<A, B, S, J2, K1 + 1>(v);
+        else dft_ab_twiddle<A, B, S, J2 + 1, 1>(v);
+    }
+}
+
+template <int R, int S>
+HDEV void dft(float2 *v);
+
+template <int A, int B, int S>
+HDEV void dft_ab(float2 *v)
+{
+#pragma unroll
+    for (int j2 = 0; j2 < B; ++j2) {
+        float2 t[A];
+#pragma unroll
+        for (int j1 = 0; j1 < A; ++j1) t[j1] = v[B * j1 + j2];
+        dft<A, S>(t);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) v[B * k1 + j2] = t[k1];
+    }
+    dft_ab_twiddle<A, B, S>(v);
+    float2 o[A * B];
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+        float2 t[B];
+#pragma unroll
+        for (int j2 = 0; j2 < B; ++j2) t[j2] = v[B * k1 + j2];
+        dft<B, S>(t);
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) o[k1 + A * k2] = t[k2];
+    }
+#pragma unroll
+    for (int k = 0; k < A * B; ++k) v[k] = o[k];
+}
+
 template <int R, int S>
 HDEV void dft(float2 *v)
 {
     if constexpr (R == 2) dft2<S>(v[0], v[1]);
+    else if constexpr (R == 6) dft_ab<2, 3, S>(v);
+    else if constexpr (R == 9) dft_ab<3, 3, S>(v);
+    else if constexpr (R == 10) dft_ab<2, 5, S>(v);
+    else if constexpr (R == 12) dft_ab<4, 3, S>(v);
+    else if constexpr (R == 14) dft_ab<2, 7, S>(v);
+    else if constexpr (R == 15) dft_ab<5, 3, S>(v);
     else if constexpr (R == 3 || R == 5 || R == 7) dft_odd<R, S>(v);
     else if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);
     else if constexpr (R == 8) dft8<S>(v);

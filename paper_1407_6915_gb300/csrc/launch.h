@@ -178,8 +178,8 @@ struct MixedArgs {
     float scale;
 };
 cudaError_t launch_mixed(int sign, const MixedArgs &a, cudaStream_t st);
-// The radix schedule for n (odd radices 7, 5, 3 first, then 8s and one 4 or
-// 2); false if n has another prime factor or is too long for one tile.
+// The radix schedule for n (the fewest stages, odd radices first); false if n
+// has a prime factor above 7 or is too long for one tile.
 bool mixed_schedule(int64_t n, int *nstages, int *radix);
 int mixed_segments_per_tile(int64_t n);
 // Factorisation and tile widths used for n.
