@@ -64,9 +64,10 @@ __global__ void __launch_bounds__(kBlueThreads) k_blue_out(const BlueArgs a)
 // coalesced store applies w and the scale to the first n points.  Each row
 // crosses HBM once each way: 8n bytes in, 8n (complex) or 4n (|X|^2) out.
 template <int LOG_M, bool BULK>
-__global__ void __launch_bounds__(256, 2) k_blue_block(const BlueBlockArgs a)
+__global__ void __launch_bounds__((BlockShape<LOG_M, kBlockLogE<LOG_M>>::T), (BlockShape<LOG_M, kBlockLogE<LOG_M>>::PER_SM))
+    k_blue_block(const BlueBlockArgs a)
 {
-    using Sh = BlockShape<LOG_M>;
+    using Sh = BlockShape<LOG_M, kBlockLogE<LOG_M>>;
     constexpr int M = 1 << LOG_M, W = 1 << Sh::LOG_W, T = Sh::T, E = Sh::E, V = E / T;
     extern __shared__ __align__(1024) float2 sm[];
     float2 *S = sm;          // staging tiles [2][W][M]
@@ -173,9 +174,9 @@ __global__ void __launch_bounds__(256, 2) k_blue_block(const BlueBlockArgs a)
 }
 
 template <int LOG_M, bool BULK>
-cudaError_t blue_block_launch(const BlueBlockArgs &a, cudaStream_t st)
+cudaError_t blue_block_launch(BlueBlockArgs a, cudaStream_t st)
 {
-    using B = BlockShape<LOG_M>;
+    using B = BlockShape<LOG_M, kBlockLogE<LOG_M>>;
     constexpr size_t smem = (size_t)(B::SLOTS + 2 * B::E) * sizeof(float2) + 2 * sizeof(uint64_t);
     auto k = k_blue_block<LOG_M, BULK>;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
@@ -188,6 +189,7 @@ cudaError_t blue_block_launch(const BlueBlockArgs &a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         per_sm = occ > 0 ? occ : 1;
     }
+    a.ntiles = (a.nseg + (1 << B::LOG_W) - 1) >> B::LOG_W;
     if (a.ntiles == 0) return cudaSuccess;
     int64_t grid = (int64_t)per_sm * device_sm_count();
     if (grid > a.ntiles) grid = a.ntiles;

@@ -48,9 +48,10 @@ __global__ void __launch_bounds__(kFrameThreads) k_frames(const FramesArgs a)
 // bins are stored from the last stage.  The samples that neighbouring frames
 // share are re-read from L2; each bin crosses HBM once.
 template <int LOG_L, bool BULK>
-__global__ void __launch_bounds__(256, 2) k_block_frames(const FramesBlockArgs a)
+__global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (BlockShape<LOG_L, kBlockLogE<LOG_L>>::PER_SM))
+    k_block_frames(const FramesBlockArgs a)
 {
-    using Sh = BlockShape<LOG_L>;
+    using Sh = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
     constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, T = Sh::T, E = Sh::E, V = E / T;
     extern __shared__ __align__(1024) float2 sm[];
     float2 *S = sm;          // staging tiles [2][W][L]
@@ -128,9 +129,9 @@ __global__ void __launch_bounds__(256, 2) k_block_frames(const FramesBlockArgs a
 }
 
 template <int LOG_L, bool BULK>
-cudaError_t block_frames_launch(const FramesBlockArgs &a, cudaStream_t st)
+cudaError_t block_frames_launch(FramesBlockArgs a, cudaStream_t st)
 {
-    using B = BlockShape<LOG_L>;
+    using B = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
     constexpr size_t smem = (size_t)(B::SLOTS + 2 * B::E) * sizeof(float2) + 2 * sizeof(uint64_t);
     auto k = k_block_frames<LOG_L, BULK>;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
@@ -143,6 +144,7 @@ cudaError_t block_frames_launch(const FramesBlockArgs &a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         per_sm = occ > 0 ? occ : 1;
     }
+    a.ntiles = (a.nframes + (1 << B::LOG_W) - 1) >> B::LOG_W;
     if (a.ntiles == 0) return cudaSuccess;
     int64_t grid = (int64_t)per_sm * device_sm_count();
     if (grid > a.ntiles) grid = a.ntiles;

@@ -22,10 +22,11 @@ int sm_count()
 }
 
 template <int LOG_L, int S, int PREC = PREC_FP32>
-cudaError_t block_t(const BlockArgs &a, cudaStream_t st)
+cudaError_t block_t(BlockArgs a, cudaStream_t st)
 {
     using B = BlockShape<LOG_L>;
     auto k = k_block<LOG_L, S, PREC>;
+    a.ntiles = (a.nseg + (1 << B::LOG_W) - 1) >> B::LOG_W;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
     int &per_sm = per_sm_dev[current_device_slot()];
     if (per_sm == 0) {
@@ -72,11 +73,6 @@ cudaError_t pass_t(const LinesArgs &a, int64_t units, cudaStream_t st)
 }
 
 }  // namespace
-
-int block_segments_per_cta(int log_n)
-{
-    return log_n >= 4 ? 1 << (12 - log_n) : 256;
-}
 
 int device_sm_count() { return sm_count(); }
 

@@ -98,9 +98,10 @@ __global__ void __launch_bounds__(kRealThreads) k_real_pre(const RealArgs a)
 // inside the tile: Z goes to the tile buffer in natural order and every
 // thread forms bin pairs (k, L - k) of one segment, written as n/2 + 1 bins.
 template <int LOG_L>
-__global__ void __launch_bounds__(256, 2) k_block_r2c(const RealBlockArgs a)
+__global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (BlockShape<LOG_L, kBlockLogE<LOG_L>>::PER_SM))
+    k_block_r2c(const RealBlockArgs a)
 {
-    using Sh = BlockShape<LOG_L>;
+    using Sh = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
     constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, E = Sh::E, T = Sh::T, V = E / T;
     constexpr int PAIRS = L / 2 + 1;
     extern __shared__ __align__(1024) float2 sm[];
@@ -181,9 +182,9 @@ __global__ void __launch_bounds__(256, 2) k_block_r2c(const RealBlockArgs a)
 }
 
 template <int LOG_L>
-cudaError_t block_r2c_t(const RealBlockArgs &a, cudaStream_t st)
+cudaError_t block_r2c_t(RealBlockArgs a, cudaStream_t st)
 {
-    using B = BlockShape<LOG_L>;
+    using B = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
     auto k = k_block_r2c<LOG_L>;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
     int &per_sm = per_sm_dev[current_device_slot()];
@@ -195,6 +196,7 @@ cudaError_t block_r2c_t(const RealBlockArgs &a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         per_sm = occ > 0 ? occ : 1;
     }
+    a.ntiles = (a.nseg + (1 << B::LOG_W) - 1) >> B::LOG_W;
     if (a.ntiles == 0) return cudaSuccess;
     int64_t grid = (int64_t)per_sm * device_sm_count();
     if (grid > a.ntiles) grid = a.ntiles;

@@ -278,12 +278,22 @@ struct BlockArgs {
     float scale;
 };
 
-template <int LOG_L>
+// 16 points per thread, 2^LOG_E points per tile (4096 with 256 threads and two
+// CTAs per SM, 2048 with 128 threads and four); lines shorter than 16 points
+// put L points in a thread and 256 lines in a tile.  Kernels that spend their
+// time between barriers take the smaller tiles where a line fits (kBlockLogE:
+// four barriers per SM that do not wait for each other: frames of 1024 points,
+// |X|^2, 235 -> 223 us for 100003, of 256 points at hop 64 215 -> 176 us for
+// 400003; real segments of 1024 samples 919 -> 881 us per 2 GiB; Bluestein
+// rows of 1009 points 647 -> 581 us for 40001).  The plain block kernel moves
+// data at the copy rate and is 5 % slower with them (1024 points, 2 GiB: 639
+// against 671 us).
+template <int LOG_L, int LOG_E = 12>
 struct BlockShape {
-    // 16 points per thread, 256 threads, 4096 points per tile; lines shorter
-    // than 16 points put L points in a thread and 256 lines in a tile.
-    static constexpr int LOG_W = LOG_L >= 4 ? 12 - LOG_L : 8;
-    static constexpr int T = 256;
+    static_assert(LOG_E == 12 || LOG_L >= 4, "short lines: 256 per tile");
+    static constexpr int LOG_W = LOG_L >= 4 ? LOG_E - LOG_L : 8;
+    static constexpr int T = 256 >> (12 - LOG_E);
+    static constexpr int PER_SM = 2 << (12 - LOG_E);
     static constexpr int E = 1 << (LOG_L + LOG_W);
     static constexpr int PS = 4;
     static constexpr int SLOTS = (smem_slots<LOG_L, LOG_W, PS>() + 1) & ~1;  // keeps the barriers 8-byte aligned

@@ -18,12 +18,14 @@ inline int current_device_slot()
 }
 
 // Single-pass segment-major tiles for n = 2^log_n <= 4096 (persistent CTAs,
-// a.ntiles tiles of block_segments_per_cta segments).  Returns the launch error.
+// a.ntiles tiles of whole segments; a.ntiles is set by the launcher).  Returns the launch error.
 // prec: PREC_FP32, or PREC_FP16 / PREC_BF16 (tensor-core radix-16 stages, n = 16, 256, 4096).
 cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cudaStream_t st);
 int device_sm_count();
-// Segments per CTA of the block kernel.
-int block_segments_per_cta(int log_n);
+// log2 of the points per tile of the frame, real-signal and Bluestein block
+// kernels for lines of 2^LOG_L points (BlockShape).
+template <int LOG_L>
+constexpr int kBlockLogE = LOG_L >= 4 && LOG_L <= 11 ? 11 : 12;
 
 // One pass of the two-pass path over lines of length 2^log_l (16..4096),
 // interleaved tiles of 2^lines_log_w(log_l) lines; `units` CTAs.

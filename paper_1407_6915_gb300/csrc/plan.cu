@@ -786,7 +786,6 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
     if (p->path == PATH_BLUESTEIN && blue_fused(p)) {
         // M <= 4096: every row on chip from chirp-in to chirp-out, one launch
         BlueBlockArgs a{};
-        const int64_t W = block_segments_per_cta(p->log_n);
         a.x = static_cast<const float2 *>(d_in);
         a.out = d_out;
         a.w = p->bw;
@@ -795,7 +794,6 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         a.err = p->d_err;
         a.n = p->n;
         a.nseg = nseg;
-        a.ntiles = (nseg + W - 1) / W;
         a.out_power = p->out_kind == FFTSEG_OUT_POWER;
         a.scale = p->scale;
         cudaError_t e = launch_blue_block(p->log_n, a, st);
@@ -882,7 +880,6 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
     if (p->path == PATH_FRAMES && frames_fused(p)) {
         // n <= 4096: windowed frames straight to their bins, one launch
         FramesBlockArgs a{};
-        const int64_t W = block_segments_per_cta(p->log_n);
         a.signal = static_cast<const float2 *>(d_in);
         a.out = d_out;
         a.window = p->fwin;
@@ -890,7 +887,6 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         a.err = p->d_err;
         a.hop = p->hop;
         a.nframes = nseg;
-        a.ntiles = (nseg + W - 1) / W;
         a.out_power = p->out_kind == FFTSEG_OUT_POWER;
         a.scale = p->inner->scale;
         cudaError_t e = launch_block_frames(p->log_n, a, st);
@@ -930,14 +926,12 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         if (p->direction == FFTSEG_FORWARD && p->inner->path == PATH_BLOCK) {
             // n/2 <= 4096: one pass, the split fused into the block kernel's tiles
             RealBlockArgs a{};
-            const int64_t W = block_segments_per_cta(p->inner->log_n);
             a.in = static_cast<const float2 *>(d_in);
             a.out = d_out;
             a.twL = p->inner->twA;
             a.tw = p->rtw;
             a.err = p->d_err;
             a.nseg = nseg;
-            a.ntiles = (nseg + W - 1) / W;
             a.out_power = power;
             a.scale = p->scale;
             cudaError_t e = launch_block_r2c(p->inner->log_n, a, st);
@@ -1024,11 +1018,9 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
     switch (p->path) {
         case PATH_BLOCK: {
             BlockArgs a{};
-            const int64_t W = block_segments_per_cta(p->log_n);
             a.in = in;
             a.out = d_out;
             a.nseg = nseg;
-            a.ntiles = (nseg + W - 1) / W;
             a.twL = p->twA;
             a.err = p->d_err;
             a.out_power = power;
