@@ -370,18 +370,25 @@ HDEV void dft_odd(float2 *v)
     float2 X0 = x0;
 #pragma unroll
     for (int k = 0; k < H; ++k) X0 = cadd(X0, A[k]);
+    if constexpr (R == 3) {  // (the sine into the last additions: one rounding less)
+        const float2 P = cfma(A[0], odd_cos<3>(1), x0), iB = mul_si<S>(B[0]);
+        constexpr float sn = odd_sin<3>(1);
+        v[1] = make_float2(iB.x * sn + P.x, iB.y * sn + P.y);
+        v[2] = make_float2(P.x - iB.x * sn, P.y - iB.y * sn);
+    } else {
 #pragma unroll
-    for (int m = 0; m < H; ++m) {
-        float2 P = x0, Q = make_float2(0.f, 0.f);
+        for (int m = 0; m < H; ++m) {
+            float2 P = x0, Q = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < H; ++k) {
-            const float c = odd_cos<R>(((m + 1) * (k + 1)) % R), sn = odd_sin<R>(((m + 1) * (k + 1)) % R);
-            P = cfma(A[k], c, P);
-            Q = cfma(B[k], sn, Q);
+            for (int k = 0; k < H; ++k) {
+                const float c = odd_cos<R>(((m + 1) * (k + 1)) % R), sn = odd_sin<R>(((m + 1) * (k + 1)) % R);
+                P = cfma(A[k], c, P);
+                Q = cfma(B[k], sn, Q);
+            }
+            const float2 iQ = mul_si<S>(Q);  // sigma i Q
+            v[m + 1] = make_float2(P.x + iQ.x, P.y + iQ.y);
+            v[R - 1 - m] = make_float2(P.x - iQ.x, P.y - iQ.y);
         }
-        const float2 iQ = mul_si<S>(Q);  // sigma i Q
-        v[m + 1] = make_float2(P.x + iQ.x, P.y + iQ.y);
-        v[R - 1 - m] = make_float2(P.x - iQ.x, P.y - iQ.y);
     }
     v[0] = X0;
 }
@@ -463,16 +470,53 @@ HDEV void dft_ab(float2 *v)
     for (int k = 0; k < A * B; ++k) v[k] = o[k];
 }
 
+// Composite radix R = A B with A, B coprime, without twiddles (the prime-factor
+// algorithm of Good and Thomas): with j = B j1 + A j2 mod R, k = k1 mod A = k2
+// mod B, w_R^{jk} = w_A^{j1 k1} w_B^{j2 k2}.
+template <int A, int B, int S>
+HDEV void dft_coprime(float2 *v)
+{
+    constexpr int R = A * B;
+    float2 y[R], o[R];
+#pragma unroll
+    for (int j2 = 0; j2 < B; ++j2) {
+        float2 t[A];
+#pragma unroll
+        for (int j1 = 0; j1 < A; ++j1) t[j1] = v[(B * j1 + A * j2) % R];
+        dft<A, S>(t);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) y[k1 * B + j2] = t[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+        dft<B, S>(y + k1 * B);
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) {
+            // k = k1 mod A = k2 mod B (a compile-time search once unrolled)
+            int k = k1;
+#pragma unroll
+            for (int i = 1; i < B; ++i)
+                if ((k1 + A * i) % B == k2) k = k1 + A * i;
+            o[k] = y[k1 * B + k2];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) v[k] = o[k];
+}
+
 template <int R, int S>
 HDEV void dft(float2 *v)
 {
     if constexpr (R == 2) dft2<S>(v[0], v[1]);
-    else if constexpr (R == 6) dft_ab<2, 3, S>(v);
+    else if constexpr (R == 6) dft_coprime<2, 3, S>(v);
     else if constexpr (R == 9) dft_ab<3, 3, S>(v);
-    else if constexpr (R == 10) dft_ab<2, 5, S>(v);
-    else if constexpr (R == 12) dft_ab<4, 3, S>(v);
-    else if constexpr (R == 14) dft_ab<2, 7, S>(v);
-    else if constexpr (R == 15) dft_ab<5, 3, S>(v);
+    else if constexpr (R == 10) dft_coprime<2, 5, S>(v);
+    else if constexpr (R == 12) dft_coprime<4, 3, S>(v);
+    else if constexpr (R == 14) dft_coprime<2, 7, S>(v);
+    else if constexpr (R == 15) dft_coprime<5, 3, S>(v);
+    else if constexpr (R == 18) dft_coprime<2, 9, S>(v);
+    else if constexpr (R == 20) dft_coprime<4, 5, S>(v);
+    else if constexpr (R == 24) dft_coprime<8, 3, S>(v);
     else if constexpr (R == 3 || R == 5 || R == 7) dft_odd<R, S>(v);
     else if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);
     else if constexpr (R == 8) dft8<S>(v);
