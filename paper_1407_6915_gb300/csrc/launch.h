@@ -3,6 +3,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <complex>
+#include <vector>
+
 #include "kernels.cuh"
 
 namespace fftseg {
@@ -165,6 +168,21 @@ struct BlueBlockArgs {
     float scale;
 };
 cudaError_t launch_blue_block(int log_m, const BlueBlockArgs &a, cudaStream_t st);
+// Bluestein rows of M = q * 1024 points in one SM each (blue_row.cu): the q for
+// length n (0: none is built), its tables, and the launch.
+struct BlueRowArgs {
+    const float2 *x;     // [nseg][n]
+    void *out;           // [nseg][n] complex64, or float32 |X|^2
+    const float2 *w;     // chirp, n values
+    const float2 *tw2, *tw1, *bhat;  // set by the launcher
+    int64_t nseg;
+    int n;
+    int out_power;
+    float scale;
+};
+int blue_row_q(int64_t n);
+void blue_row_tables(int q, const std::vector<std::complex<double>> &b, std::vector<float2> &h);
+cudaError_t launch_blue_row(int q, const float2 *tables, BlueRowArgs a, cudaStream_t st);
 // Lengths n = 2^a 3^b 5^c 7^d <= 4096 (not powers of two) in one pass
 // (k_mixed.cu): mixed-radix Stockham stages over tiles of whole segments.
 constexpr int kMixMaxStages = 16;

@@ -521,7 +521,7 @@ int64_t launches_per_exec(fftseg_plan p, int64_t nseg)
         case PATH_FOURSTEP: return p->ilv_log_r ? 2 * ((nseg + p->work_segs - 1) / p->work_segs) : 1;
         case PATH_MIXED: return 1;
         case PATH_BLUESTEIN: {
-            if (blue_fused(p)) return 1;
+            if (p->blue_q || blue_fused(p)) return 1;
             int64_t k = 0;
             for (int64_t s0 = 0; s0 < nseg; s0 += p->rchunk) {
                 const int64_t c = nseg - s0 < p->rchunk ? nseg - s0 : p->rchunk;
@@ -780,6 +780,20 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         }
         cudaError_t e = launch_mixed(p->direction, a, st);
         if (e != cudaSuccess) return cuda_error(e, "mixed-radix kernel launch");
+        count_launches(1);
+        return FFTSEG_OK;
+    }
+    if (p->path == PATH_BLUESTEIN && p->blue_q) {
+        BlueRowArgs a{};
+        a.x = static_cast<const float2 *>(d_in);
+        a.out = d_out;
+        a.w = p->bw;
+        a.nseg = nseg;
+        a.n = (int)p->n;
+        a.out_power = p->out_kind == FFTSEG_OUT_POWER;
+        a.scale = p->scale;
+        cudaError_t e = launch_blue_row(p->blue_q, p->bhat, a, st);
+        if (e != cudaSuccess) return cuda_error(e, "Bluestein row kernel launch");
         count_launches(1);
         return FFTSEG_OK;
     }
@@ -1353,6 +1367,22 @@ int create_frames(fftseg_plan *out, int64_t n, int64_t hop, int window, int64_t 
 // 18.6 for 256 MiB and 23.0 for L2-sized 32 MiB chunks.
 constexpr int kBlueChunkMB = 1024;
 
+// w (rounded once) and b = conj(w) placed cyclically over M points, divided by M
+void blue_chirp(int64_t n, int64_t M, int direction, std::vector<float2> &w, std::vector<std::complex<double>> &b)
+{
+    const double pi = 3.141592653589793238462643383279, inv_m = 1.0 / (double)M;
+    w.resize((size_t)n);
+    b.assign((size_t)M, 0.0);
+    for (int64_t m = 0; m < n; ++m) {
+        const int64_t e2 = (int64_t)(((unsigned __int128)m * (unsigned __int128)m) % (unsigned __int128)(2 * n));
+        const double a = pi * ((double)e2 / (double)n);
+        const double c = cos(a), sn = (double)direction * sin(a);
+        w[(size_t)m] = make_float2((float)c, (float)sn);
+        b[(size_t)m] = std::complex<double>(c * inv_m, -sn * inv_m);
+        if (m > 0) b[(size_t)(M - m)] = b[(size_t)m];
+    }
+}
+
 int create_bluestein(fftseg_plan *out, int64_t n, int64_t batch, int direction, int norm, int out_kind,
                      unsigned flags)
 {
@@ -1378,6 +1408,32 @@ int create_bluestein(fftseg_plan *out, int64_t n, int64_t batch, int direction, 
     p->bm = M;
     if (norm == FFTSEG_NORM_BACKWARD) p->scale = direction == FFTSEG_INVERSE ? (float)(1.0 / (double)n) : 1.f;
     else if (norm == FFTSEG_NORM_ORTHO) p->scale = (float)(1.0 / sqrt((double)n));
+    // n = 2049..12288: rows of q * 1024 points in one SM each, in one launch
+    // (an asked-for schedule, and FFTSEG_FLAG_BLUESTEIN, which asks for
+    // power-of-two rows, keep the passes over rows of M points)
+    const int q = flags & (kPathFlags | FFTSEG_FLAG_AUTOTUNE | FFTSEG_FLAG_BLUESTEIN) ? 0 : blue_row_q(n);
+    if (q) {
+        const int64_t m = (int64_t)q * 1024;
+        std::vector<float2> w, h;
+        std::vector<std::complex<double>> b;
+        blue_chirp(n, m, direction, w, b);
+        blue_row_tables(q, b, h);
+        p->blue_q = q;
+        p->bm = m;
+        int rc = upload(&p->bw, w);
+        if (rc == FFTSEG_OK) rc = upload(&p->bhat, h);
+        if (rc == FFTSEG_OK) {
+            e = cudaMalloc((void **)&p->d_err, sizeof(int));
+            if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
+            if (e != cudaSuccess) rc = cuda_error(e, "cudaMalloc(status flag)");
+        }
+        if (rc != FFTSEG_OK) {
+            free_plan(p);
+            return rc;
+        }
+        *out = p;
+        return FFTSEG_OK;
+    }
     int64_t cs = ((int64_t)env_int("FFTSEG_BLUE_CHUNK_MB", kBlueChunkMB, 1, 4096) << 20) / (M * 8);
     if (cs < 1) cs = 1;
     if (cs > 65535) cs = 65535;
@@ -1399,18 +1455,10 @@ int create_bluestein(fftseg_plan *out, int64_t n, int64_t batch, int direction, 
         rc = fftseg_plan_create(&p->inner2, M, cs, FFTSEG_INVERSE, FFTSEG_NORM_NONE, FFTSEG_PREC_FP32,
                                 FFTSEG_OUT_COMPLEX, iflags);
     if (rc == FFTSEG_OK) {
-        const double pi = 3.141592653589793238462643383279;
-        std::vector<float2> w((size_t)n), b((size_t)M, make_float2(0.f, 0.f));
-        const double inv_m = 1.0 / (double)M;
-        for (int64_t m = 0; m < n; ++m) {
-            const int64_t e2 = (int64_t)(((unsigned __int128)m * (unsigned __int128)m) % (unsigned __int128)(2 * n));
-            const double a = pi * ((double)e2 / (double)n);
-            const double c = cos(a), sn = (double)direction * sin(a);
-            w[(size_t)m] = make_float2((float)c, (float)sn);
-            const float2 cb = make_float2((float)(c * inv_m), (float)(-sn * inv_m));  // conj(w) / M
-            b[(size_t)m] = cb;
-            if (m > 0) b[(size_t)(M - m)] = cb;
-        }
+        std::vector<float2> w, b((size_t)M);
+        std::vector<std::complex<double>> bd;
+        blue_chirp(n, M, direction, w, bd);
+        for (int64_t m = 0; m < M; ++m) b[(size_t)m] = make_float2((float)bd[(size_t)m].real(), (float)bd[(size_t)m].imag());
         rc = upload(&p->bw, w);
         float2 *bdev = nullptr;
         if (rc == FFTSEG_OK) rc = upload(&bdev, b);
@@ -1630,7 +1678,7 @@ int fftseg_plan_info(fftseg_plan p, int64_t info[6])
 {
     if (!p || !info) return set_error(FFTSEG_E_INVALID, "plan_info: NULL argument");
     info[0] = p->path;
-    info[1] = p->path == PATH_MIXED ? p->n : int64_t(1) << p->log_n1;
+    info[1] = p->path == PATH_MIXED ? p->n : p->blue_q ? p->bm : int64_t(1) << p->log_n1;
     info[2] = (p->path == PATH_BLOCK || p->path == PATH_REAL || p->path == PATH_FRAMES ||
                p->path == PATH_BLUESTEIN || p->path == PATH_MIXED)
                   ? 1
@@ -1640,7 +1688,8 @@ int fftseg_plan_info(fftseg_plan p, int64_t info[6])
               : p->path == PATH_REAL ? (p->rwork ? p->rchunk * (p->n / 2) * 8 : 0)
                                     : p->work ? p->work_segs * p->n * 8
                                               : (p->ring ? (int64_t)p->ring_nr * p->ring_cs * p->n * 8 : 0);
-    info[4] = (p->path == PATH_REAL || p->path == PATH_FRAMES || p->path == PATH_BLUESTEIN) ? p->rchunk
+    info[4] = p->blue_q ? p->batch
+              : (p->path == PATH_REAL || p->path == PATH_FRAMES || p->path == PATH_BLUESTEIN) ? p->rchunk
               : p->path == PATH_MIXED ? mixed_segments_per_tile(p->n)
               : p->work ? p->work_segs : p->ring_cs;
     info[5] = launches_per_exec(p, p->batch);

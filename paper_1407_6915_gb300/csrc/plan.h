@@ -86,6 +86,7 @@ struct fftseg_plan_s {
     int mix_radix[16] = {}, mix_twoff[16] = {};
     float2 *bw = nullptr, *bhat = nullptr;
     int64_t bm = 0;
+    int blue_q = 0;  // rows of blue_q * 1024 points in one SM each (bhat: that kernel's tables)
     // fftseg_stream phase split of the last call (ms)
     double phases[6] = {0, 0, 0, 0, 0, 0};
     // fftseg_exec_host device staging (owned; released with the plan)
