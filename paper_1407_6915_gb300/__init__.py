@@ -32,7 +32,7 @@ FILE_DIRECT, FILE_KEEP = 0x1, 0x2
 
 WINDOW_RECT, WINDOW_HANN = 0, 1
 PATH_NAMES = {0: "block", 1: "cluster", 2: "two-pass", 3: "tensor-core", 4: "four-step", 5: "real",
-              6: "frames", 7: "bluestein", 8: "mixed-radix"}
+              6: "frames", 7: "bluestein", 8: "mixed-radix", 9: "one-sm"}
 
 OK, E_INVALID, E_NOMEM, E_CUDA, E_IO, E_PARTIAL, E_TIMEOUT, E_UNSUPPORTED = 0, -1, -2, -3, -4, -5, -6, -7
 

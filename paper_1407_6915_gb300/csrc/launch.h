@@ -63,6 +63,17 @@ cudaError_t launch_cluster_blue_inv(int log_m, int log_c, const ClusterArgs &a, 
 // Bluestein rows of M = 2^log_m points: the forward transform of the chirped
 // input rows of a.bl_n samples (read directly, zero past them) into a.out.
 cudaError_t launch_cluster_blue_fwd(int log_m, int log_c, const ClusterArgs &a, cudaStream_t st);
+// Segments of 2^14 points in one SM each (one_sm.cu): its tables, and the launch.
+struct OneSmArgs {
+    const float2 *in;
+    void *out;
+    const float2 *tw;
+    int64_t nseg;
+    int out_power;
+    float scale;
+};
+void one_sm_tables(std::vector<float2> &h);
+cudaError_t launch_one_sm(int sign, const OneSmArgs &a, cudaStream_t st);
 // Factorisation used for n: *log_n1, *log_n2, default cluster size *log_c.
 bool cluster_shape(int log_n, int log_c_req, int *log_n1, int *log_n2, int *log_c);
 

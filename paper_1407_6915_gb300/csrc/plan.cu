@@ -206,6 +206,7 @@ void free_plan(fftseg_plan p)
     cudaFree(p->fwin);
     cudaFree(p->win_row);
     cudaFree(p->win_col);
+    cudaFree(p->one_sm);
     if (p->host_stage && p->host_stage_free) p->host_stage_free(p->host_stage);
     cudaFree(p->twA);
     cudaFree(p->twB);
@@ -485,6 +486,13 @@ int build_fp32(fftseg_plan p)
         p->log_c = lc;
         if ((rc = stage_table(&p->twA, int64_t(1) << l1))) return rc;
         if ((rc = stage_table(&p->twB, int64_t(1) << l2))) return rc;
+        if (ln == 14 && want_c == 0) {
+            // (the cluster tables stay: real-signal and Bluestein plans fold their
+            // passes into the cluster kernel)
+            std::vector<float2> h;
+            one_sm_tables(h);
+            if ((rc = upload(&p->one_sm, h))) return rc;
+        }
         return fourstep_table(&p->tw4a, p->n, int64_t(1) << l1, 1, int64_t(1) << l2);
     }
     p->path = PATH_TWOPASS;
@@ -1045,6 +1053,13 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
             return FFTSEG_OK;
         }
         case PATH_CLUSTER: {
+            if (p->one_sm) {
+                const OneSmArgs o{in, d_out, p->one_sm, nseg, power, p->scale};
+                e = launch_one_sm(sign, o, st);
+                if (e != cudaSuccess) return cuda_error(e, "one-SM kernel launch");
+                count_launches(1);
+                return FFTSEG_OK;
+            }
             ClusterArgs a{};
             const int64_t N1 = int64_t(1) << p->log_n1, N2 = int64_t(1) << p->log_n2;
             const uint32_t WA = (uint32_t)(N2 >> p->log_c);
@@ -1677,9 +1692,9 @@ int fftseg_exec(fftseg_plan p, const void *d_in, void *d_out, fftseg_stream_t st
 int fftseg_plan_info(fftseg_plan p, int64_t info[6])
 {
     if (!p || !info) return set_error(FFTSEG_E_INVALID, "plan_info: NULL argument");
-    info[0] = p->path;
-    info[1] = p->path == PATH_MIXED ? p->n : p->blue_q ? p->bm : int64_t(1) << p->log_n1;
-    info[2] = (p->path == PATH_BLOCK || p->path == PATH_REAL || p->path == PATH_FRAMES ||
+    info[0] = p->one_sm ? PATH_ONE_SM : p->path;
+    info[1] = p->path == PATH_MIXED || p->one_sm ? p->n : p->blue_q ? p->bm : int64_t(1) << p->log_n1;
+    info[2] = (p->one_sm || p->path == PATH_BLOCK || p->path == PATH_REAL || p->path == PATH_FRAMES ||
                p->path == PATH_BLUESTEIN || p->path == PATH_MIXED)
                   ? 1
                   : int64_t(1) << p->log_n2;

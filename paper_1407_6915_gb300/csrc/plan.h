@@ -20,7 +20,8 @@ enum Path {
     PATH_REAL = 5,
     PATH_FRAMES = 6,
     PATH_BLUESTEIN = 7,
-    PATH_MIXED = 8
+    PATH_MIXED = 8,
+    PATH_ONE_SM = 9  // reported only: a cluster plan whose segments run in one SM each
 };
 
 }  // namespace fftseg
@@ -86,6 +87,7 @@ struct fftseg_plan_s {
     int mix_radix[16] = {}, mix_twoff[16] = {};
     float2 *bw = nullptr, *bhat = nullptr;
     int64_t bm = 0;
+    float2 *one_sm = nullptr;  // n = 2^14 by default: the tables of the kernel with a segment per SM
     int blue_q = 0;  // rows of blue_q * 1024 points in one SM each (bhat: that kernel's tables)
     // fftseg_stream phase split of the last call (ms)
     double phases[6] = {0, 0, 0, 0, 0, 0};

@@ -82,6 +82,7 @@ std::vector<unsigned> candidates(int log_n, int prec)
         c.push_back(0);
         return c;
     }
+    if (log_n == 14) c.push_back(0);  // a segment per SM
     for (int lc = 1; lc <= 4; ++lc) {
         int l1, l2, got;
         if (log_n <= 17 && cluster_shape(log_n, lc, &l1, &l2, &got) && got == lc)
