@@ -282,9 +282,8 @@ struct BlockArgs {
 // CTAs per SM, 2048 with 128 threads and four); lines shorter than 16 points
 // put L points in a thread and 256 lines in a tile.  Kernels that spend their
 // time between barriers take the smaller tiles where a line fits (kBlockLogE:
-// four barriers per SM that do not wait for each other: frames of 1024 points,
-// |X|^2, 235 -> 223 us for 100003, of 256 points at hop 64 215 -> 176 us for
-// 400003; real segments of 1024 samples 919 -> 881 us per 2 GiB; Bluestein
+// four barriers per SM that do not wait for each other: frames of 2048
+// points and shorter than 256; real segments of 1024 samples 919 -> 881 us per 2 GiB; Bluestein
 // rows of 1009 points 647 -> 581 us for 40001).  The plain block kernel moves
 // data at the copy rate and is 5 % slower with them (1024 points, 2 GiB: 639
 // against 671 us).

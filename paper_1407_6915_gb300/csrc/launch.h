@@ -146,6 +146,7 @@ struct FramesBlockArgs {
     void *out;             // [nframes][n] complex64, or float32 |X|^2
     const float *window;   // n values, or null for the rectangular window
     const float2 *twL;     // stage tables of the n-point line
+    const float2 *twW;     // n = 256, 512, 1024: w_n^{j r} at [r][32], r < n / 32
     int *err;              // set to 1 if a copy never completed
     int64_t hop, nframes, ntiles;
     int out_power;

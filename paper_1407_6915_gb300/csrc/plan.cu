@@ -206,6 +206,7 @@ void free_plan(fftseg_plan p)
     cudaFree(p->fwin);
     cudaFree(p->win_row);
     cudaFree(p->win_col);
+    cudaFree(p->ftw);
     cudaFree(p->one_sm);
     if (p->host_stage && p->host_stage_free) p->host_stage_free(p->host_stage);
     cudaFree(p->twA);
@@ -906,6 +907,7 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         a.out = d_out;
         a.window = p->fwin;
         a.twL = p->inner->twA;
+        a.twW = p->ftw;
         a.err = p->d_err;
         a.hop = p->hop;
         a.nframes = nseg;
@@ -1344,6 +1346,11 @@ int create_frames(fftseg_plan *out, int64_t n, int64_t hop, int window, int64_t 
             rc = upload(&p->win_row, r);
             if (rc == FFTSEG_OK) rc = upload(&p->win_col, c);
         }
+    }
+    if (rc == FFTSEG_OK && n >= 256 && n <= 1024) {
+        std::vector<float2> h((size_t)n);
+        for (int64_t r = 0; r < n / 32; ++r) host_roots(h.data() + 32 * r, 32, n, r);
+        rc = upload(&p->ftw, h);
     }
     if (rc == FFTSEG_OK && window == FFTSEG_WINDOW_HANN && !p->frames_wl) {
         // periodic Hann window, w[j] = (1 - cos(2 pi j / n)) / 2, evaluated in double

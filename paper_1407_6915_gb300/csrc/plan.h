@@ -71,6 +71,7 @@ struct fftseg_plan_s {
     int64_t hop = 0;
     int window = 0;
     float *fwin = nullptr;  // the window, n values (null: rectangular)
+    float2 *ftw = nullptr;  // n = 256, 512, 1024: w_n^{j r}, [n / 32][32]
     // frame plans on the lane-line kernel (hop a multiple of N2, complex
     // output): frames go straight from the signal into its column tiles, the
     // Hann window from the factors win_row[j1] = (cos, sin)(2 pi j1 / N1),
