@@ -36,20 +36,23 @@ constexpr int kRow = 1024;  // the inner 32 x 32 points
 template <int Q>
 struct BlueRowShape {
     static constexpr int M = Q * kRow;
-    static constexpr int T = Q <= 6 ? 128 : Q <= 12 ? 256 : 512, PER_SM = 512 / T;
+    // (Q = 24: 768 radix-32 butterflies in two full rounds, 286 -> 268 us at n = 12281)
+    static constexpr int T = Q <= 6 ? 128 : Q <= 12 ? 256 : Q == 24 ? 384 : 512, PER_SM = 512 / T;
     static constexpr int A = (Q + 3) / 4;  // w_M^{j r}: r = 4 a + b, two factors
     static constexpr int H = Q / 2 + 1;    // points j + 1024 r < n have r < H (2 n - 1 <= M)
     static constexpr size_t SMEM = (size_t)(M + kRow) * sizeof(float2);
     static_assert(PER_SM * (SMEM + 1024) <= 228 * 1024, "rows per SM");
 };
 
-// The radix-Q butterfly.  Radix 20 as 4 x 5 with twiddles: half of S1's points
-// are zero, whole inputs of its first radix-4 butterflies, and it needs fewer
-// registers than the prime-factor form here (n = 10007: 291 against 311 us).
+// The radix-Q butterfly.  Radix 10 and 20 as 2 x 5 and 4 x 5 with twiddles: half
+// of S1's points are zero, whole inputs of their first butterflies, and they need
+// fewer registers than the prime-factor form here (n = 10007: 291 against 311 us,
+// n = 5003: 272 against 308).
 template <int Q, int S>
 FDEV void row_dft(float2 *v)
 {
-    if constexpr (Q == 20) dft_ab<4, 5, S>(v);
+    if constexpr (Q == 10) dft_ab<2, 5, S>(v);
+    else if constexpr (Q == 20) dft_ab<4, 5, S>(v);
     else dft<Q, S>(v);
 }
 
