@@ -140,9 +140,28 @@ def check(status, what="fftseg"):
     return status
 
 
+# torch, once an entry point has needed it (importing the binding does not), and
+# its raw current-stream query where it has one
+_torch = None
+_raw_stream = None
+
+
+def _load_torch():
+    global _torch, _raw_stream
+    import torch
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if not hasattr(torch._C, "_cuda_getDevice"):
+        _raw_stream = None
+    _torch = torch
+    return torch
+
+
 def _stream_handle(stream):
     if stream is None:
-        import torch
+        torch = _torch or _load_torch()
+        # (the raw handle: a torch.cuda.Stream made per call costs as much as the launch)
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -218,8 +237,10 @@ class Plan:
 
     def exec_ptr(self, d_in: int, d_out: int, nseg: int = None, stream=None) -> None:
         """Raw-pointer form of fftseg_exec_n (asynchronous on `stream`)."""
-        nseg = self.batch if nseg is None else nseg
-        check(lib().fftseg_exec_n(self._h, d_in, d_out, nseg, _stream_handle(stream)), "fftseg_exec")
+        rc = (_lib or lib()).fftseg_exec_n(self._h, d_in, d_out, self.batch if nseg is None else nseg,
+                                           _stream_handle(stream))
+        if rc:
+            check(rc, "fftseg_exec")
 
     def exec_host(self, h_in, h_out, nseg=None, chunk_segments=0) -> None:
         """fftseg_exec_host with this plan alone (host tensors or addresses)."""
@@ -230,18 +251,16 @@ class Plan:
         (allocated if None).  Complex plans: x complex64 [.., n].  Real-signal
         plans (FLAG_REAL): forward x float32 [.., n] -> complex64 (or float32
         power) [.., n/2 + 1]; inverse x complex64 [.., n/2 + 1] -> float32 [.., n]."""
-        import torch
+        torch = _torch or _load_torch()
         if not (x.is_cuda and x.is_contiguous()):
             raise ValueError("fftseg.Plan.exec wants a contiguous CUDA tensor")
-        real = bool(self.flags & FLAG_REAL)
-        if real and self.direction == FORWARD:
-            want, seg_in, seg_out = torch.float32, self.n, self.n // 2 + 1
-            out_dt = torch.float32 if self.out_kind == OUT_POWER else torch.complex64
-        elif real:
-            want, seg_in, seg_out, out_dt = torch.complex64, self.n // 2 + 1, self.n, torch.float32
-        else:
+        out_dt = torch.float32 if self.out_kind == OUT_POWER else torch.complex64
+        if not self.flags & FLAG_REAL:
             want, seg_in, seg_out = torch.complex64, self.n, self.n
-            out_dt = torch.float32 if self.out_kind == OUT_POWER else torch.complex64
+        elif self.direction == FORWARD:
+            want, seg_in, seg_out = torch.float32, self.n, self.n // 2 + 1
+        else:
+            want, seg_in, seg_out, out_dt = torch.complex64, self.n // 2 + 1, self.n, torch.float32
         if x.dtype != want:
             raise ValueError("fftseg.Plan.exec wants %s input for this plan" % want)
         nseg = (x.numel() // seg_in) if nseg is None else nseg
@@ -359,7 +378,7 @@ class FramePlan(Plan):
         """Frames of the complex64 device signal x (contiguous): the first
         nseg frames (default: every whole frame, at most batch) -> out
         [nframes][n] (complex64, or float32 |X|^2)."""
-        import torch
+        torch = _torch or _load_torch()
         if not (x.is_cuda and x.is_contiguous() and x.dtype == torch.complex64):
             raise ValueError("fftseg.FramePlan.exec wants a contiguous complex64 CUDA tensor")
         avail = self.frames_in(x.numel())
