@@ -283,10 +283,10 @@ struct BlockArgs {
 // put L points in a thread and 256 lines in a tile.  Kernels that spend their
 // time between barriers take the smaller tiles where a line fits (kBlockLogE:
 // four barriers per SM that do not wait for each other: frames of 2048
-// points and shorter than 256; real segments of 1024 samples 919 -> 881 us per 2 GiB; Bluestein
-// rows of 1009 points 647 -> 581 us for 40001).  The plain block kernel moves
-// data at the copy rate and is 5 % slower with them (1024 points, 2 GiB: 639
-// against 671 us).
+// points and shorter than 256; real segments of 1024 samples 919 -> 881 us per
+// 2 GiB; Bluestein rows of 1009 points 647 -> 581 us for 40001).  The plain block
+// kernel moves data at the copy rate and is 5 % slower with them on large
+// batches (1024 points, 2 GiB: 639 against 671 us), faster on small ones.
 template <int LOG_L, int LOG_E = 12>
 struct BlockShape {
     static_assert(LOG_E == 12 || LOG_L >= 4, "short lines: 256 per tile");
@@ -302,11 +302,11 @@ struct BlockShape {
 // One tile of whole segments, already in shared memory (Pb, dense [c][i]):
 // W segments from segment line0 on (those at or past nseg are not stored).
 // With tensor-core stages tc->stage must point into Pb (this warp's 4 KB).
-template <int LOG_L, int S, int PREC = PREC_FP32>
+template <int LOG_L, int S, int PREC = PREC_FP32, int LOG_E = 12>
 FDEV void block_tile(const float2 *Pb, float2 *X, const float2 *__restrict__ twL, int64_t line0, int64_t nseg,
                      void *out, int out_power, float scale, const TcCtx *tc)
 {
-    using Sh = BlockShape<LOG_L>;
+    using Sh = BlockShape<LOG_L, LOG_E>;
     constexpr int L = 1 << LOG_L, T = Sh::T, V = Sh::E / T;
     float2 v[V];
     gather<LOG_L, Sh::LOG_W, false, T, 0>(v, [&](int c, int i) { return Pb[(c << LOG_L) + i]; });
@@ -325,10 +325,11 @@ FDEV void block_tile(const float2 *Pb, float2 *X, const float2 *__restrict__ twL
     });
 }
 
-template <int LOG_L, int S, int PREC = PREC_FP32>
-__global__ void __launch_bounds__(256, PREC == PREC_FP32 ? 2 : 1) k_block(const BlockArgs a)
+template <int LOG_L, int S, int PREC = PREC_FP32, int LOG_E = 12>
+__global__ void __launch_bounds__((BlockShape<LOG_L, LOG_E>::T), PREC == PREC_FP32 ? (BlockShape<LOG_L, LOG_E>::PER_SM) : 1)
+    k_block(const BlockArgs a)
 {
-    using Sh = BlockShape<LOG_L>;
+    using Sh = BlockShape<LOG_L, LOG_E>;
     constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, E = Sh::E, T = Sh::T, V = E / T;
     // TMA destinations first: the dynamic shared base is 1024-byte aligned and
     // each prefetch buffer is a multiple of 1024 bytes
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(256, PREC == PREC_FP32 ? 2 : 1) k_block(const 
         if (u + gridDim.x < a.ntiles) issue(u + gridDim.x, b ^ 1);
         mbar_wait(&bar[b], (k >> 1) & 1, a.err);
         if constexpr (PREC != PREC_FP32) tc.stage = P + b * E + (threadIdx.x >> 5) * 512;
-        block_tile<LOG_L, S, PREC>(P + b * E, X, a.twL, u * W, a.nseg, a.out, a.out_power, scale, &tc);
+        block_tile<LOG_L, S, PREC, LOG_E>(P + b * E, X, a.twL, u * W, a.nseg, a.out, a.out_power, scale, &tc);
         __syncthreads();  // P[b] fully read before it is refilled two tiles on
     }
 }

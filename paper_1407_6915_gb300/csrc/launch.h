@@ -26,7 +26,8 @@ inline int current_device_slot()
 cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cudaStream_t st);
 int device_sm_count();
 // log2 of the points per tile of the frame, real-signal and Bluestein block
-// kernels for lines of 2^LOG_L points (BlockShape).
+// kernels (and of the plain one for small batches) for lines of 2^LOG_L points
+// (BlockShape).
 template <int LOG_L>
 constexpr int kBlockLogE = LOG_L >= 4 && LOG_L <= 11 ? 11 : 12;
 

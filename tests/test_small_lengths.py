@@ -1,4 +1,4 @@
-"""The mixed-radix kernel's composite in-register butterflies (6, 9, 10, 12, 14,
+"""Short lengths.  The mixed-radix kernel's composite in-register butterflies (6, 9, 10, 12, 14,
 15) and their compile-time rotations, compiled for the host from the kernels'
 own header against the direct DFT in double, and every smooth length's schedule
 on the GPU path: lengths whose stages use each of them, one and two stages, the
@@ -86,3 +86,22 @@ def test_every_radix_and_tile_edge(n, direction):
         y = fs.Plan(n, B, direction).exec(torch.from_numpy(x).cuda())
         torch.cuda.synchronize()
         assert rel_l2(y.cpu().numpy(), oracle.dft(x, direction)) <= tol_fp32(n), (n, B)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [16, 64, 1024, 2048])
+def test_block_tile_sizes_give_the_same_bits(n):
+    # batches on either side of the 2^22 points where the block kernel changes its
+    # tiles: a segment's bits do not depend on them, nor on a ragged last tile
+    torch = pytest.importorskip("torch")
+    import paper_1407_6915_gb300 as fs
+
+    B = (1 << 22) // n
+    x = torch.view_as_complex(torch.rand((B + 1, n, 2), device="cuda").sub_(0.5))
+    plan = fs.Plan(n, B + 1, fs.FORWARD, fs.NORM_ORTHO)
+    large, small = plan.exec(x), plan.exec(x[:B])
+    odd = plan.exec(x[:3])
+    torch.cuda.synchronize()
+    assert torch.equal(large[:B], small) and torch.equal(large[:3], odd)
+    host = x[-2:].cpu().numpy()
+    assert rel_l2(large[-2:].cpu().numpy(), oracle.fft(host, fs.FORWARD, fs.NORM_ORTHO)) <= tol_fp32(n)
