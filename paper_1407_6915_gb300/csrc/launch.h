@@ -69,6 +69,7 @@ struct OneSmArgs {
     const float2 *in;
     void *out;
     const float2 *tw;
+    int *err;  // set when a copy never completed
     int64_t nseg;
     int out_power;
     float scale;

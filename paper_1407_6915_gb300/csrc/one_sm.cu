@@ -7,9 +7,11 @@
 //   S2  radix 32 over b, times w_512^{c k_b}
 //   S3  radix 16 over c: X[k_a + 32 k_b + 1024 k_c], to global memory
 // Three barriers and 32 bytes of shared-memory traffic per point, and no traffic
-// between SMs.  4001 segments: 199 us (0.79 of the copy rate), against 249 us (0.63)
+// between SMs.  4001 segments: 186 us (0.84 of the copy rate), against 249 us (0.63)
 // for the 4-CTA cluster kernel, which waits for its all-to-all exchange between
-// SMs.  (Four stages of radix 16, 16, 16, 4 with 1024 threads of 64 registers
+// SMs.  22 of the next segment's 32 rows are copied into the shared memory left
+// over while a segment runs (199 us with all of them read when it starts).  (Four
+// stages of radix 16, 16, 16, 4 with 1024 threads of 64 registers
 // measured 266 us: half as much shared-memory traffic again and a barrier more,
 // and with one CTA per SM nothing overlaps a stage.)
 //
@@ -25,13 +27,29 @@ namespace {
 
 constexpr int kN = 1 << 14, kT = 512;
 constexpr int kTw2 = 10 * 512, kTw = kTw2 + 31 * 16;  // w_n^{j r} factors, then w_512^{c r}
+constexpr int kAhead = 22;  // rows of 512 points of the next segment copied in while this one runs
+constexpr size_t kSmem = (size_t)(kN + 31 * 16 + kAhead * 512) * sizeof(float2) + sizeof(uint64_t);
 
 template <int S>
 __global__ void __launch_bounds__(kT, 1) k_one_sm(const OneSmArgs a)
 {
     extern __shared__ float2 sm[];
     const int tid = threadIdx.x;
-    float2 *const T2 = sm + kN;  // [r-1][c]
+    float2 *const P = sm + kN;              // rows ahead
+    float2 *const T2 = P + kAhead * 512;    // [r-1][c]
+    uint64_t *const bar = reinterpret_cast<uint64_t *>(T2 + 31 * 16);
+    constexpr uint32_t AHEAD_BYTES = kAhead * 512 * sizeof(float2);
+    auto ahead = [&](int64_t s) {
+        mbar_expect_tx(bar, AHEAD_BYTES);
+        tma_load_1d(P, a.in + s * kN, AHEAD_BYTES, bar);
+    };
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
+        if ((int64_t)blockIdx.x < a.nseg) ahead(blockIdx.x);
+    }
+    uint32_t par = 0;
+    __syncthreads();
     if (tid < 31 * 16) T2[tid] = __ldg(a.tw + kTw2 + tid);  // (S2 reads it after S1's barrier)
     const int a2 = tid >> 4, c2 = tid & 15, o2 = 512 * a2 + (c2 ^ (a2 & 15));
     const int a3 = tid & 31, x3 = a3 & 15, o3 = 512 * a3;
@@ -40,7 +58,11 @@ __global__ void __launch_bounds__(kT, 1) k_one_sm(const OneSmArgs a)
         {  // S1
             const float2 *const x = a.in + s * kN + tid;
 #pragma unroll
-            for (int r = 0; r < 32; ++r) v[r] = x[512 * r];
+            for (int r = kAhead; r < 32; ++r) v[r] = x[512 * r];
+            mbar_wait(bar, par, a.err);
+            par ^= 1;
+#pragma unroll
+            for (int r = 0; r < kAhead; ++r) v[r] = P[512 * r + tid];
             float2 wb[8], wa[4];  // w_n^{j b}, w_n^{8 j a}
 #pragma unroll
             for (int i = 1; i < 8; ++i) wb[i] = __ldg(a.tw + (i - 1) * 512 + tid);
@@ -54,8 +76,11 @@ __global__ void __launch_bounds__(kT, 1) k_one_sm(const OneSmArgs a)
             }
         }
         __syncthreads();
-        if (tid == 0 && s + gridDim.x < a.nseg)  // the next segment on its way to L2
-            prefetch_l2_bulk(a.in + (s + gridDim.x) * kN, kN * (uint32_t)sizeof(float2));
+        if (tid == 0 && s + gridDim.x < a.nseg) {  // the next segment: the rows ahead, the others to L2
+            fence_proxy_async();
+            ahead(s + gridDim.x);
+            prefetch_l2_bulk(a.in + (s + gridDim.x) * kN + kAhead * 512, (32 - kAhead) * 512 * (uint32_t)sizeof(float2));
+        }
         {  // S2
 #pragma unroll
             for (int r = 0; r < 32; ++r) v[r] = sm[o2 + 16 * r];
@@ -98,17 +123,16 @@ __global__ void __launch_bounds__(kT, 1) k_one_sm(const OneSmArgs a)
 template <int S>
 cudaError_t one_sm_t(const OneSmArgs &a, cudaStream_t st)
 {
-    constexpr size_t SMEM = (size_t)(kN + kTw - kTw2) * sizeof(float2);
     auto k = k_one_sm<S>;
     static bool configured_dev[kMaxDevices] = {};  // per instantiation and device
     bool &configured = configured_dev[current_device_slot()];
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         if (e != cudaSuccess) return e;
         configured = true;
     }
     const int64_t sms = device_sm_count();
-    k<<<(unsigned)(a.nseg < sms ? a.nseg : sms), kT, SMEM, st>>>(a);
+    k<<<(unsigned)(a.nseg < sms ? a.nseg : sms), kT, kSmem, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -1056,7 +1056,7 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         }
         case PATH_CLUSTER: {
             if (p->one_sm) {
-                const OneSmArgs o{in, d_out, p->one_sm, nseg, power, p->scale};
+                const OneSmArgs o{in, d_out, p->one_sm, p->d_err, nseg, power, p->scale};
                 e = launch_one_sm(sign, o, st);
                 if (e != cudaSuccess) return cuda_error(e, "one-SM kernel launch");
                 count_launches(1);
