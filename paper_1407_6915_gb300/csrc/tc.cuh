@@ -28,6 +28,19 @@ namespace fftseg {
 
 enum { PREC_FP32 = 0, PREC_FP16 = 1, PREC_BF16 = 2 };
 
+// cos(2 pi q / 16), from the rounded first-quadrant values (the same floats as
+// a double-precision evaluation, whose few hundred FP64 instructions per thread
+// took about 16 us of every launch on this GPU's FP64 units)
+FDEV float cos16(int q)
+{
+    q &= 15;
+    q = q > 8 ? 16 - q : q;
+    const int a = q > 4 ? 8 - q : q;
+    const float c = a == 0 ? 1.f : a == 1 ? kC16a : a == 2 ? kC8 : a == 3 ? kC16b : 0.f;
+    return q > 4 ? -c : c;
+}
+FDEV float sin16(int q) { return cos16(q - 4); }
+
 struct TcCtx {
     uint32_t bh[16];  // F hi fragments: [(ks * 4 + nt) * 2 + q]
     uint32_t bl[16];  // F lo fragments
@@ -85,9 +98,7 @@ FDEV void tc_init(TcCtx &tc, float2 *stage)
                 for (int e = 0; e < 2; ++e) {
                     const int k = 16 * ks + 2 * t + 8 * q + e;
                     const int j = k >> 1, im_in = k & 1;
-                    double sd, cd;
-                    sincospi(2.0 * (double)((j * m) & 15) / 16.0, &sd, &cd);
-                    const float c = (float)cd, s = (float)(S * sd);
+                    const float c = cos16(j * m), s = (float)S * sin16(j * m);
                     f[e] = im_in == 0 ? (im_out == 0 ? c : s) : (im_out == 0 ? -s : c);
                 }
                 float la, lb;

@@ -54,9 +54,7 @@ struct WlTcF {
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                     const int m = g + 8 * mt, r = t + 4 * (2 * kt + q);
-                    double sd, cd;
-                    sincospi((double)((r * m) & 15) / 8.0, &sd, &cd);
-                    const float c = (float)cd, s = (float)(S * sd);
+                    const float c = cos16(r * m), s = (float)S * sin16(r * m);
                     float la, lb;
                     h[mt][kt][2 * q] = pack_hi<PREC>(c, -s, la, lb);  // row re(m)
                     l[mt][kt][2 * q] = pack_lo<PREC>(la, lb);
