@@ -181,18 +181,141 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (Bl
     }
 }
 
+// Inverse real segments of n = 2L <= 8192 points in one pass: tiles of whole
+// segments' bins (L + 1 each, contiguous) arrive by bulk copies, the join above
+// runs in place on the tile (each pair (k, L - k) belongs to one thread), then
+// the L-point Stockham FFT, written as n samples.  A bulk copy must start and
+// end on 16 bytes, and a segment has an odd number of 8-byte bins: a tile's
+// copy is widened to 16-byte boundaries (one bin of a neighbouring segment at
+// most), except at the end of the batch, where the last segment's bin X[L] is
+// read from global memory instead.  Bound by memory: 2^29 samples of
+// n = 256 .. 2048 take 678 .. 762 us, n = 8192 862 us (643 at the copy rate);
+// a join pass before the transform, through a 512 MiB intermediate, moved each
+// bin through memory twice more (1909 .. 1392, 1425 us; 2^23 samples of 1024:
+// 37 us, now 22).
 template <int LOG_L>
-cudaError_t block_r2c_t(RealBlockArgs a, cudaStream_t st)
+struct C2rShape : BlockShape<LOG_L, kBlockLogE<LOG_L>> {
+    using B = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
+    static constexpr int BUF = (B::E + (1 << B::LOG_W) + 2 + 15) & ~15;  // bins per buffer, in whole 128 bytes
+    static constexpr size_t SMEM = (size_t)(B::SLOTS + 2 * BUF) * sizeof(float2) + 2 * sizeof(uint64_t);
+};
+
+template <int LOG_L>
+__global__ void __launch_bounds__((C2rShape<LOG_L>::T), (C2rShape<LOG_L>::PER_SM)) k_block_c2r(const RealBlockArgs a)
+{
+    using Sh = C2rShape<LOG_L>;
+    constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, E = Sh::E, T = Sh::T, V = E / T, BUF = Sh::BUF;
+    extern __shared__ __align__(1024) float2 sm[];
+    float2 *P = sm;
+    float2 *X = sm + 2 * BUF;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(X + Sh::SLOTS);
+    const int tid = threadIdx.x;
+    if (smem_u32(P) & 127) {
+        if (tid == 0) atomicOr(a.err, 2);
+        return;
+    }
+    if (tid == 0) {
+        mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    // tile u: bins [first, last) of the batch, copied from the even bin at or
+    // before first to the even bin at or after last (before, at the batch's end)
+    auto first_bin = [&](int64_t u) { return u * W * (int64_t)(L + 1); };
+    auto copy_from = [&](int64_t u) { return first_bin(u) & ~(int64_t)1; };
+    auto copy_bytes = [&](int64_t u) {
+        const int64_t total = a.nseg * (int64_t)(L + 1);
+        int64_t end = (first_bin(u + 1) + 1) & ~(int64_t)1;
+        if (end > total) end = total & ~(int64_t)1;
+        return (uint32_t)((end - copy_from(u)) * (int64_t)sizeof(float2));
+    };
+    grid_launch_dependents();
+    if (tid == 0)
+        for (int64_t u = blockIdx.x, q = 0; q < 2 && u < a.ntiles; ++q, u += gridDim.x)
+            prefetch_l2_bulk(a.in + copy_from(u), copy_bytes(u));
+    grid_dependency_wait();
+    auto issue = [&](int64_t u, int b) {
+        if (tid == 0) {
+            const uint32_t bytes = copy_bytes(u);
+            fence_proxy_async();
+            mbar_expect_tx(&bar[b], bytes);
+            tma_load_1d(P + b * BUF, a.in + copy_from(u), bytes, &bar[b]);
+        }
+    };
+    int64_t u = blockIdx.x;
+    if (u < a.ntiles) issue(u, 0);
+    float *out = static_cast<float *>(a.out);
+    for (int k = 0; u < a.ntiles; u += gridDim.x, ++k) {
+        const int b = k & 1;
+        if (u + gridDim.x < a.ntiles) issue(u + gridDim.x, b ^ 1);
+        mbar_wait(&bar[b], (k >> 1) & 1, a.err);
+        const int64_t line0 = u * W;
+        float2 *Pb = P + b * BUF + (first_bin(u) & 1);
+        // the join: pairs (kk, L - kk), kk = 0 .. L/2 - 1; kk = 0 also does L/2.
+        // All reads of a thread come before its writes (segments past the
+        // batch hold stale values, which are not stored)
+        {
+            constexpr int NP = E / 2 / T > 0 ? E / 2 / T : 1;
+            float2 A[NP], C[NP], w[NP];
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                const int p = tid + q * T, c = p >> (LOG_L - 1), kk = p & (L / 2 - 1);
+                A[q] = Pb[c * (L + 1) + kk];
+                C[q] = Pb[c * (L + 1) + L - kk];
+                w[q] = __ldg(a.tw + kk);
+            }
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                const int p = tid + q * T, c = p >> (LOG_L - 1), kk = p & (L / 2 - 1);
+                float2 *Z = Pb + c * (L + 1);
+                if (kk == 0) {
+                    if (line0 + c == a.nseg - 1) C[q] = __ldcg(a.in + a.nseg * (int64_t)(L + 1) - 1);
+                    A[q].y = 0.f;  // the imaginary parts of the real bins X[0] and X[L] do not enter
+                    C[q].y = 0.f;
+                }
+                const float2 B = conjf2(C[q]);
+                const float2 d = cmul(conjf2(w[q]), make_float2(A[q].x - B.x, A[q].y - B.y));
+                const float2 z = scalef2(make_float2(A[q].x + B.x - d.y, A[q].y + B.y + d.x), a.scale);
+                float2 m;
+                if (kk == 0) {  // Z[L/2] from X[L/2] with itself
+                    m = Z[L / 2];
+                    const float2 B2 = conjf2(m);
+                    const float2 d2 = cmul(conjf2(__ldg(a.tw + L / 2)), make_float2(m.x - B2.x, m.y - B2.y));
+                    m = scalef2(make_float2(m.x + B2.x - d2.y, m.y + B2.y + d2.x), a.scale);
+                } else {
+                    const float2 B2 = conjf2(A[q]);
+                    const float2 d2 = cmul(make_float2(-w[q].x, -w[q].y), make_float2(C[q].x - B2.x, C[q].y - B2.y));
+                    m = scalef2(make_float2(C[q].x + B2.x - d2.y, C[q].y + B2.y + d2.x), a.scale);
+                }
+                Z[kk] = z;
+                Z[kk == 0 ? L / 2 : L - kk] = m;
+            }
+        }
+        __syncthreads();
+        float2 v[V];
+        gather<LOG_L, Sh::LOG_W, false, T, 0>(v, [&](int c, int i) { return Pb[c * (L + 1) + i]; });
+        run_stages<LOG_L, Sh::LOG_W, false, 1, T, Sh::PS, 0, false>(v, X, a.twL);
+        scatter_last<LOG_L, Sh::LOG_W, false, T>(v, [&](int c, int i, float2 x) {
+            if (line0 + c < a.nseg) reinterpret_cast<float2 *>(out)[(line0 + c) * L + i] = x;
+        });
+        __syncthreads();  // P[b] and X read in full before they are reused
+    }
+}
+
+template <int LOG_L, bool INVERSE>
+cudaError_t block_real_t(RealBlockArgs a, cudaStream_t st)
 {
     using B = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
-    auto k = k_block_r2c<LOG_L>;
+    constexpr size_t SMEM = INVERSE ? C2rShape<LOG_L>::SMEM : B::SMEM;
+    auto k = INVERSE ? k_block_c2r<LOG_L> : k_block_r2c<LOG_L>;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
     int &per_sm = per_sm_dev[current_device_slot()];
     if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
         if (e != cudaSuccess) return e;
         int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, B::T, B::SMEM);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, B::T, SMEM);
         if (e != cudaSuccess) return e;
         per_sm = occ > 0 ? occ : 1;
     }
@@ -200,29 +323,33 @@ cudaError_t block_r2c_t(RealBlockArgs a, cudaStream_t st)
     if (a.ntiles == 0) return cudaSuccess;
     int64_t grid = (int64_t)per_sm * device_sm_count();
     if (grid > a.ntiles) grid = a.ntiles;
-    return launch_programmatic(k, (unsigned)grid, B::T, B::SMEM, st, a);
+    return launch_programmatic(k, (unsigned)grid, B::T, SMEM, st, a);
+}
+
+template <bool INVERSE>
+cudaError_t block_real(int log_l, const RealBlockArgs &a, cudaStream_t st)
+{
+    switch (log_l) {
+        case 1: return block_real_t<1, INVERSE>(a, st);
+        case 2: return block_real_t<2, INVERSE>(a, st);
+        case 3: return block_real_t<3, INVERSE>(a, st);
+        case 4: return block_real_t<4, INVERSE>(a, st);
+        case 5: return block_real_t<5, INVERSE>(a, st);
+        case 6: return block_real_t<6, INVERSE>(a, st);
+        case 7: return block_real_t<7, INVERSE>(a, st);
+        case 8: return block_real_t<8, INVERSE>(a, st);
+        case 9: return block_real_t<9, INVERSE>(a, st);
+        case 10: return block_real_t<10, INVERSE>(a, st);
+        case 11: return block_real_t<11, INVERSE>(a, st);
+        case 12: return block_real_t<12, INVERSE>(a, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace
 
-cudaError_t launch_block_r2c(int log_l, const RealBlockArgs &a, cudaStream_t st)
-{
-    switch (log_l) {
-        case 1: return block_r2c_t<1>(a, st);
-        case 2: return block_r2c_t<2>(a, st);
-        case 3: return block_r2c_t<3>(a, st);
-        case 4: return block_r2c_t<4>(a, st);
-        case 5: return block_r2c_t<5>(a, st);
-        case 6: return block_r2c_t<6>(a, st);
-        case 7: return block_r2c_t<7>(a, st);
-        case 8: return block_r2c_t<8>(a, st);
-        case 9: return block_r2c_t<9>(a, st);
-        case 10: return block_r2c_t<10>(a, st);
-        case 11: return block_r2c_t<11>(a, st);
-        case 12: return block_r2c_t<12>(a, st);
-        default: return cudaErrorInvalidValue;
-    }
-}
+cudaError_t launch_block_r2c(int log_l, const RealBlockArgs &a, cudaStream_t st) { return block_real<false>(log_l, a, st); }
+cudaError_t launch_block_c2r(int log_l, const RealBlockArgs &a, cudaStream_t st) { return block_real<true>(log_l, a, st); }
 
 cudaError_t launch_real(bool post, bool power, RealArgs a, int64_t nseg, cudaStream_t st)
 {

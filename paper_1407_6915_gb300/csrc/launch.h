@@ -130,6 +130,7 @@ struct RealBlockArgs {
     float scale;
 };
 cudaError_t launch_block_r2c(int log_l, const RealBlockArgs &a, cudaStream_t st);
+cudaError_t launch_block_c2r(int log_l, const RealBlockArgs &a, cudaStream_t st);  // in: bins, out: samples
 // Overlapping segments (frames.cu): windowed frames f = samples
 // [f*hop, f*hop + n) of the signal into [nframes][n] complex64.
 struct FramesArgs {

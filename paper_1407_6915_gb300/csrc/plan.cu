@@ -87,11 +87,10 @@ bool frames_fused(const fftseg_plan_s *p)
            p->inner->precision == FFTSEG_PREC_FP32;
 }
 
-// Forward real-signal plans whose n/2-point complex transform runs on the
-// block or the cluster kernel split the spectrum inside that kernel (one
-// pass, no intermediate); inverse ones join the bins inside the cluster
-// kernel up to n/2 = 2^14 for batches of at most 64 MiB of samples.  (The
-// fused join reads its bins with plain loads, a point and its mirror:
+// Real-signal plans whose n/2-point complex transform runs on the block kernel
+// split or join the bins inside that kernel (one pass, no intermediate); so do
+// forward ones on the cluster kernel, and inverse ones there up to n/2 = 2^14
+// for batches of at most 64 MiB of samples.  (The cluster kernel's join reads its bins with plain loads, a point and its mirror:
 // measured on GB300 at n = 2^14 and 2^15 over 4 GiB, 0.37 and 0.35 of the
 // copy peak against 0.39 and 0.37 in 512 MiB chunks, at 256 MiB 0.35 / 0.34
 // against 0.37 / 0.36, and for 37 segments 9.1 / 12.4 us against
@@ -101,9 +100,10 @@ bool frames_fused(const fftseg_plan_s *p)
 bool real_fused(const fftseg_plan_s *p)
 {
     if (p->path != PATH_REAL || !p->inner) return false;
+    if (p->inner->path == PATH_BLOCK) return true;
     if (p->direction == FFTSEG_INVERSE)
         return p->inner->path == PATH_CLUSTER && p->inner->log_n <= 14 && p->batch * p->n * 4 <= (int64_t(64) << 20);
-    return p->inner->path == PATH_BLOCK || p->inner->path == PATH_CLUSTER;
+    return p->inner->path == PATH_CLUSTER;
 }
 int ilog2(int64_t n)
 {
@@ -947,8 +947,9 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
     if (p->path == PATH_REAL) {
         const int64_t M = p->n / 2;
         const bool power = p->out_kind == FFTSEG_OUT_POWER;
-        if (p->direction == FFTSEG_FORWARD && p->inner->path == PATH_BLOCK) {
-            // n/2 <= 4096: one pass, the split fused into the block kernel's tiles
+        if (p->inner->path == PATH_BLOCK) {
+            // n/2 <= 4096: one pass, the split or the join fused into the block kernel's tiles
+            const bool fwd = p->direction == FFTSEG_FORWARD;
             RealBlockArgs a{};
             a.in = static_cast<const float2 *>(d_in);
             a.out = d_out;
@@ -958,7 +959,7 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
             a.nseg = nseg;
             a.out_power = power;
             a.scale = p->scale;
-            cudaError_t e = launch_block_r2c(p->inner->log_n, a, st);
+            cudaError_t e = fwd ? launch_block_r2c(p->inner->log_n, a, st) : launch_block_c2r(p->inner->log_n, a, st);
             if (e != cudaSuccess) return cuda_error(e, "real-signal block kernel launch");
             count_launches(1);
             return FFTSEG_OK;
