@@ -35,6 +35,26 @@ FDEV float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y,
 FDEV float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
 FDEV float2 scalef2(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 
+// X[k] and X[M - k] (scaled) from Z[k], C = Z[(M - k) mod M] and w = w_n^k
+FDEV void split_pair(float2 A, float2 C, float2 w, float scale, float2 &xk, float2 &xm)
+{
+    const float2 B = conjf2(C);
+    const float2 fe = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y + B.y));
+    const float2 fo = make_float2(0.5f * (A.y - B.y), -0.5f * (A.x - B.x));  // -i (A - B) / 2
+    const float2 wfo = cmul(w, fo);
+    xk = scalef2(make_float2(fe.x + wfo.x, fe.y + wfo.y), scale);
+    xm = scalef2(make_float2(fe.x - wfo.x, -(fe.y - wfo.y)), scale);  // conj(Fe - w Fo)
+}
+
+// Z[k] (scaled) from A = X[k], C = X[M - k] and v = conj(w_n^k):
+// (A + conj(C)) + i v (A - conj(C)).  Z[M - k] is the same of (C, A, -w_n^k).
+FDEV float2 join_bin(float2 A, float2 C, float2 v, float scale)
+{
+    const float2 B = conjf2(C);
+    const float2 d = cmul(v, make_float2(A.x - B.x, A.y - B.y));
+    return scalef2(make_float2(A.x + B.x - d.y, A.y + B.y + d.x), scale);
+}
+
 // One block covers kRealThreads pairs of one segment: block b -> segment
 // b / bps, pairs (b % bps) * kRealThreads + threadIdx.x.
 template <bool POWER>
@@ -46,13 +66,8 @@ __global__ void __launch_bounds__(kRealThreads) k_real_post(const RealArgs a)
     const int M = a.m;
     if (k > M / 2) return;
     const float2 *Z = a.zin + s * M;
-    const float2 A = Z[k];
-    const float2 B = conjf2(Z[(M - k) & (M - 1)]);
-    const float2 fe = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y + B.y));
-    const float2 fo = make_float2(0.5f * (A.y - B.y), -0.5f * (A.x - B.x));  // -i (A - B) / 2
-    const float2 wfo = cmul(__ldg(a.tw + k), fo);
-    const float2 xk = scalef2(make_float2(fe.x + wfo.x, fe.y + wfo.y), a.scale);
-    const float2 xm = scalef2(make_float2(fe.x - wfo.x, -(fe.y - wfo.y)), a.scale);  // conj(Fe - w Fo)
+    float2 xk, xm;
+    split_pair(Z[k], Z[(M - k) & (M - 1)], __ldg(a.tw + k), a.scale, xk, xm);
     const int64_t o = s * (M + 1);
     if (POWER) {
         float *P = static_cast<float *>(a.out) + o;
@@ -80,30 +95,25 @@ __global__ void __launch_bounds__(kRealThreads) k_real_pre(const RealArgs a)
     }
     const float2 w = __ldg(a.tw + k);  // w_n^k (forward value); conj(w) = exp(+2 pi i k / n)
     float2 *Z = static_cast<float2 *>(a.out) + s * M;
-    {  // Z[k] = (A + conj(C)) + i conj(w) (A - conj(C))
-        const float2 B = conjf2(C);
-        const float2 d = cmul(conjf2(w), make_float2(A.x - B.x, A.y - B.y));
-        Z[k] = scalef2(make_float2(A.x + B.x - d.y, A.y + B.y + d.x), a.scale);
-    }
-    if (k != 0 && 2 * k != M) {  // Z[M - k] from the same pair: conj(w_n^{M-k}) = -w_n^k
-        const float2 B = conjf2(A);
-        const float2 d = cmul(make_float2(-w.x, -w.y), make_float2(C.x - B.x, C.y - B.y));
-        Z[M - k] = scalef2(make_float2(C.x + B.x - d.y, C.y + B.y + d.x), a.scale);
-    }
+    Z[k] = join_bin(A, C, conjf2(w), a.scale);
+    if (k != 0 && 2 * k != M) Z[M - k] = join_bin(C, A, make_float2(-w.x, -w.y), a.scale);
 }
 
 // Forward real segments of n = 2L <= 8192 points in one pass: the block
 // kernel's persistent CTAs and bulk-copied tiles of whole segments (the L
 // complex values of each), the L-point Stockham FFT, then the split above
 // inside the tile: Z goes to the tile buffer in natural order and every
-// thread forms bin pairs (k, L - k) of one segment, written as n/2 + 1 bins.
+// thread forms bin pairs (k, L - k), written as n/2 + 1 bins.  Bound by memory
+// and, up to n = 256, by the stores' partial lines: 2^29 samples of n = 256 ..
+// 4096 take 673 .. 809 us, n = 8192 872 us (643 at the copy rate).  Eight pairs
+// are read before the first is stored: one pair at a time, each waited for its
+// shared-memory reads, 757 .. 906 and 1023 us.
 template <int LOG_L>
 __global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (BlockShape<LOG_L, kBlockLogE<LOG_L>>::PER_SM))
     k_block_r2c(const RealBlockArgs a)
 {
     using Sh = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
     constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, E = Sh::E, T = Sh::T, V = E / T;
-    constexpr int PAIRS = L / 2 + 1;
     extern __shared__ __align__(1024) float2 sm[];
     float2 *P = sm;
     float2 *X = sm + 2 * E;
@@ -155,26 +165,35 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (Bl
         scatter_last<LOG_L, Sh::LOG_W, false, T>(v, [&](int c, int i, float2 x) { Pb[(c << LOG_L) + i] = x; });
         __syncthreads();
         const int64_t line0 = u * W;
-        for (int p = tid; p < W * PAIRS; p += T) {
-            const int c = p / PAIRS, kk = p - c * PAIRS;
+        // pairs (kk, L - kk), kk = 0 .. L/2 - 1; kk = 0 also does L/2.  A thread's
+        // reads all come before its first store
+        constexpr int NP = E / 2 / T;
+        float2 A[NP], C[NP], w[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            const int p = tid + q * T, c = p >> (LOG_L - 1), kk = p & (L / 2 - 1);
+            A[q] = Pb[(c << LOG_L) + kk];
+            C[q] = Pb[(c << LOG_L) + ((L - kk) & (L - 1))];
+            w[q] = __ldg(a.tw + kk);
+        }
+        auto store = [&](int64_t o, float2 x) {
+            if (a.out_power) static_cast<float *>(a.out)[o] = x.x * x.x + x.y * x.y;
+            else static_cast<float2 *>(a.out)[o] = x;
+        };
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            const int p = tid + q * T, c = p >> (LOG_L - 1), kk = p & (L / 2 - 1);
             const int64_t seg = line0 + c;
             if (seg >= a.nseg) continue;
-            const float2 A = Pb[(c << LOG_L) + kk];
-            const float2 B = conjf2(Pb[(c << LOG_L) + ((L - kk) & (L - 1))]);
-            const float2 fe = make_float2(0.5f * (A.x + B.x), 0.5f * (A.y + B.y));
-            const float2 fo = make_float2(0.5f * (A.y - B.y), -0.5f * (A.x - B.x));
-            const float2 wfo = cmul(__ldg(a.tw + kk), fo);
-            const float2 xk = scalef2(make_float2(fe.x + wfo.x, fe.y + wfo.y), a.scale);
-            const float2 xm = scalef2(make_float2(fe.x - wfo.x, -(fe.y - wfo.y)), a.scale);
             const int64_t o = seg * (L + 1);
-            if (a.out_power) {
-                float *Q = static_cast<float *>(a.out) + o;
-                Q[kk] = xk.x * xk.x + xk.y * xk.y;
-                if (2 * kk != L) Q[L - kk] = xm.x * xm.x + xm.y * xm.y;
-            } else {
-                float2 *Q = static_cast<float2 *>(a.out) + o;
-                Q[kk] = xk;
-                if (2 * kk != L) Q[L - kk] = xm;
+            float2 xk, xm;
+            split_pair(A[q], C[q], w[q], a.scale, xk, xm);
+            store(o + kk, xk);
+            store(o + L - kk, xm);
+            if (kk == 0) {
+                const float2 m = Pb[(c << LOG_L) + L / 2];
+                split_pair(m, m, __ldg(a.tw + L / 2), a.scale, xk, xm);
+                store(o + L / 2, xk);
             }
         }
         __syncthreads();  // P[b] and X read in full before they are reused
@@ -256,7 +275,7 @@ __global__ void __launch_bounds__((C2rShape<LOG_L>::T), (C2rShape<LOG_L>::PER_SM
         // All reads of a thread come before its writes (segments past the
         // batch hold stale values, which are not stored)
         {
-            constexpr int NP = E / 2 / T > 0 ? E / 2 / T : 1;
+            constexpr int NP = E / 2 / T;
             float2 A[NP], C[NP], w[NP];
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
@@ -274,20 +293,9 @@ __global__ void __launch_bounds__((C2rShape<LOG_L>::T), (C2rShape<LOG_L>::PER_SM
                     A[q].y = 0.f;  // the imaginary parts of the real bins X[0] and X[L] do not enter
                     C[q].y = 0.f;
                 }
-                const float2 B = conjf2(C[q]);
-                const float2 d = cmul(conjf2(w[q]), make_float2(A[q].x - B.x, A[q].y - B.y));
-                const float2 z = scalef2(make_float2(A[q].x + B.x - d.y, A[q].y + B.y + d.x), a.scale);
-                float2 m;
-                if (kk == 0) {  // Z[L/2] from X[L/2] with itself
-                    m = Z[L / 2];
-                    const float2 B2 = conjf2(m);
-                    const float2 d2 = cmul(conjf2(__ldg(a.tw + L / 2)), make_float2(m.x - B2.x, m.y - B2.y));
-                    m = scalef2(make_float2(m.x + B2.x - d2.y, m.y + B2.y + d2.x), a.scale);
-                } else {
-                    const float2 B2 = conjf2(A[q]);
-                    const float2 d2 = cmul(make_float2(-w[q].x, -w[q].y), make_float2(C[q].x - B2.x, C[q].y - B2.y));
-                    m = scalef2(make_float2(C[q].x + B2.x - d2.y, C[q].y + B2.y + d2.x), a.scale);
-                }
+                const float2 z = join_bin(A[q], C[q], conjf2(w[q]), a.scale);
+                const float2 m = kk == 0 ? join_bin(Z[L / 2], Z[L / 2], conjf2(__ldg(a.tw + L / 2)), a.scale)
+                                         : join_bin(C[q], A[q], make_float2(-w[q].x, -w[q].y), a.scale);
                 Z[kk] = z;
                 Z[kk == 0 ? L / 2 : L - kk] = m;
             }

@@ -284,7 +284,7 @@ struct BlockArgs {
 // time between barriers take the smaller tiles where a line fits (kBlockLogE:
 // four barriers per SM that do not wait for each other: frames of 2048
 // points and shorter than 256; real segments of 1024 samples 919 -> 881 us per
-// 2 GiB; Bluestein rows of 1009 points 647 -> 581 us for 40001).  The plain block
+// 2 GiB (807 now); Bluestein rows of 1009 points 647 -> 581 us for 40001).  The plain block
 // kernel moves data at the copy rate and is 5 % slower with them on large
 // batches (1024 points, 2 GiB: 639 against 671 us), faster on small ones.
 template <int LOG_L, int LOG_E = 12>

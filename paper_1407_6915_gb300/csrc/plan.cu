@@ -90,7 +90,8 @@ bool frames_fused(const fftseg_plan_s *p)
 // Real-signal plans whose n/2-point complex transform runs on the block kernel
 // split or join the bins inside that kernel (one pass, no intermediate); so do
 // forward ones on the cluster kernel, and inverse ones there up to n/2 = 2^14
-// for batches of at most 64 MiB of samples.  (The cluster kernel's join reads its bins with plain loads, a point and its mirror:
+// for batches of at most 64 MiB of samples.  (The cluster kernel's join reads
+// its bins with plain loads, a point and its mirror:
 // measured on GB300 at n = 2^14 and 2^15 over 4 GiB, 0.37 and 0.35 of the
 // copy peak against 0.39 and 0.37 in 512 MiB chunks, at 256 MiB 0.35 / 0.34
 // against 0.37 / 0.36, and for 37 segments 9.1 / 12.4 us against
