@@ -12,18 +12,19 @@
 // write and one read of the tile in shared memory and a barrier, which is what
 // the kernel spends its time on (1000 = 10 10 10 in three stages instead of
 // 5 5 5 8 in four, with the last stage's bins going from registers straight
-// to the output: 200 -> 174 us for 40001 segments).  Odd radices come first:
-// their Ns = 1 stage stores with an odd stride, which no two lanes of a
-// half-warp share a bank pair with.  (Stage outputs padded against the bank
-// conflicts of the other stages, or the butterflies' slots from a table,
-// measured no faster: the index arithmetic or the table's latency took what
-// they gave.)
+// to the output: 200 -> 174 us for 40001 segments).  Among those it is the one,
+// with its tile, that a model of the stages' bank conflicts and of the threads
+// left idle finds fastest (mixed_cost below): a first stage of radix 16 stores
+// at a stride of 16 points, all in one bank pair, so 1536 runs as 6 16 16 and
+// not 16 16 6 (2^25 points: 142 us against 228).  (Stage outputs padded against
+// the bank conflicts of the other stages, or the butterflies' slots from a
+// table, measured no faster: the index arithmetic or the table's latency took
+// what they gave.)
 //
 // Each CTA (persistent) takes tiles of floor(E / n) whole segments, E = 2048
-// with 128 threads and four CTAs per SM up to n = 2048 (four barriers that do
-// not wait for each other: 1000 points 174 -> 162 us), else 4096 with 256
-// threads and two.  The next tile is copied in with one bulk copy (or 8-byte cp.async
-// copies by every thread) while the current one runs its stages, ping-ponging
+// with 128 threads and four CTAs per SM (four barriers that do not wait for
+// each other: 1000 points 174 -> 162 us), or 4096 with 256 threads and two
+// where the segment is longer or fills the smaller tile badly (1029).  The next tile is copied in with one bulk copy while the current one runs its stages, ping-ponging
 // between two shared buffers with one barrier per stage.  Stage twiddles are
 // read through the read-only cache.
 #include "engine.cuh"
@@ -34,8 +35,7 @@ namespace fftseg {
 
 namespace {
 
-constexpr int kMixEMax = 4096;  // the longest segment
-int mix_tile(int64_t n) { return n <= 2048 ? 2048 : 4096; }  // points per tile buffer
+constexpr int kMixEMax = 4096;  // the longest segment, and the larger tile
 template <int E>
 constexpr int kMixThreads = E / 16;
 
@@ -118,13 +118,19 @@ __global__ void __launch_bounds__(kMixThreads<E>, 8192 / E) k_mixed(const __grid
         const int64_t left = a.nseg - t * spt;
         return (int)(left < spt ? left : spt);
     };
-    // A tile whose bytes start on a 16-byte boundary and are a multiple of 16
-    // (an even number of points) arrives by one bulk copy issued by thread 0
-    // and completed on an mbarrier; otherwise every thread issues 8-byte
-    // cp.async copies.
+    // A tile arrives by one bulk copy issued by thread 0 and completed on an
+    // mbarrier.  The copy must start and end on 16 bytes, two points: for odd n
+    // it starts or ends up to one point outside the tile (which still fits the
+    // buffer: a tile that is full has an even number of points), except at the
+    // end of an odd batch, whose last point thread 0 reads by itself.
     __shared__ __align__(8) uint64_t bar[2];
-    auto bulk_ok = [&](int64_t t) -> bool {
-        return ((t * spt * (int64_t)n) & 1) == 0 && ((count_of(t) * n) & 1) == 0;
+    const int64_t total = a.nseg * (int64_t)n;
+    auto copy_from = [&](int64_t t) { return (t * spt * (int64_t)n) & ~(int64_t)1; };
+    auto copy_bytes = [&](int64_t t) {
+        int64_t end = t * spt * (int64_t)n + count_of(t) * n;
+        end = (end + 1) & ~(int64_t)1;
+        if (end > total) end = total & ~(int64_t)1;
+        return (uint32_t)((end - copy_from(t)) * (int64_t)sizeof(float2));
     };
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
@@ -138,40 +144,30 @@ __global__ void __launch_bounds__(kMixThreads<E>, 8192 / E) k_mixed(const __grid
     grid_launch_dependents();
     if (threadIdx.x == 0)
         for (int64_t t = blockIdx.x, q = 0; q < 2 && t < a.ntiles; ++q, t += gridDim.x)
-            if (bulk_ok(t))
-                prefetch_l2_bulk(a.in + t * spt * (int64_t)n, (uint32_t)(count_of(t) * n * sizeof(float2)));
+            prefetch_l2_bulk(a.in + copy_from(t), copy_bytes(t));
     grid_dependency_wait();
     uint32_t phase = 0;  // bit b: parity of the next completion of bar[b]
     auto load = [&](int64_t t, float2 *dst, int b) {
-        const float2 *src = a.in + t * spt * (int64_t)n;
-        const int count = count_of(t) * n;
-        if (bulk_ok(t)) {
-            if (threadIdx.x == 0) {
-                fence_proxy_async();  // this buffer's earlier generic accesses before the copy
-                mbar_expect_tx(&bar[b], (uint32_t)(count * sizeof(float2)));
-                tma_load_1d(dst, src, (uint32_t)(count * sizeof(float2)), &bar[b]);
-            }
-        } else {
-            for (int e = threadIdx.x; e < count; e += T) cp_async8(dst + e, src + e, 8);
+        if (threadIdx.x == 0) {
+            const uint32_t bytes = copy_bytes(t);
+            fence_proxy_async();  // this buffer's earlier generic accesses before the copy
+            mbar_expect_tx(&bar[b], bytes);
+            tma_load_1d(dst, a.in + copy_from(t), bytes, &bar[b]);
         }
     };
     int64_t t = blockIdx.x;
     if (t < a.ntiles) load(t, buf0, 0);
-    cp_async_commit();
     int cur = 0;
     for (; t < a.ntiles; t += gridDim.x) {
         const int64_t tn = t + gridDim.x;
         if (tn < a.ntiles) load(tn, cur ? buf0 : buf1, cur ^ 1);
-        cp_async_commit();
-        cp_async_wait<1>();  // this tile's copies (the group before the one just issued)
-        if (bulk_ok(t)) {
-            mbar_wait(&bar[cur], (phase >> cur) & 1, a.err);
-            phase ^= 1u << cur;
-        }
+        mbar_wait(&bar[cur], (phase >> cur) & 1, a.err);
+        phase ^= 1u << cur;
+        const int64_t o0 = t * spt * (int64_t)n;
+        float2 *src = (cur ? buf1 : buf0) + (o0 & 1), *dst = buf2;
+        if (threadIdx.x == 0 && t == a.ntiles - 1 && (total & 1)) src[total - 1 - o0] = a.in[total - 1];
         __syncthreads();
         const int cnt = count_of(t);
-        float2 *src = cur ? buf1 : buf0, *dst = buf2;
-        const int64_t o0 = t * spt * (int64_t)n;
         MixOut mo{nullptr, a.scale, a.out_power};
         for (int st = 0; st < a.nstages; ++st) {
             if (st == a.nstages - 1)
@@ -202,7 +198,6 @@ __global__ void __launch_bounds__(kMixThreads<E>, 8192 / E) k_mixed(const __grid
         }
         cur ^= 1;
     }
-    cp_async_wait<0>();
 }
 
 template <int S, int E>
@@ -230,52 +225,109 @@ cudaError_t mixed_t(const MixedArgs &a, cudaStream_t st)
 
 }  // namespace
 
-int mixed_segments_per_tile(int64_t n) { return n <= kMixEMax ? (int)(mix_tile(n) / n) : 0; }
-
 namespace {
 
-// The fewest stages whose radices multiply to m, each at most `top`; among
-// those the smallest largest radix.  Radices come out in falling order.
-bool mixed_search(int64_t m, int top, int left, int *radix, int depth)
+// Wavefronts of a half-warp's 8-byte shared-memory access: the most of its
+// different slots that share one of the 16 bank pairs.
+int half_warp_wavefronts(const int *slot, int lanes)
 {
-    static const int R[] = {16, 15, 14, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
-    if (left == 0) return m == 1;
-    for (int r : R) {
-        if (r > top || m % r) continue;
-        radix[depth] = r;
-        if (mixed_search(m / r, r, left - 1, radix, depth + 1)) return true;
+    int most = 0;
+    for (int i = 0; i < lanes; ++i) {
+        int w = 1;  // different slots in this slot's bank pair, counted from the last one on
+        for (int k = i + 1; k < lanes; ++k) {
+            if (((slot[k] ^ slot[i]) & 15) != 0) continue;
+            bool again = false;
+            for (int l = i; l < k && !again; ++l) again = slot[l] == slot[k];
+            w += !again;
+        }
+        if (w > most) most = w;
     }
-    return false;
+    return most;
+}
+
+// Modelled time of a schedule, per point: what the kernel spends on a tile's
+// stages, fitted to 26 lengths from 90 to 4050 (all within 14 %, us per 2^26
+// points): 20 per butterfly point in the threads' passes, idle threads of a
+// last pass included; 12.1 per wavefront of the stages' shared-memory accesses
+// (in units of a half-warp), taken from the first four half-warps of a stage's
+// butterflies; 379 per thread and stage for the barriers and the start.  (The
+// constant 44 of the fit, the same for all, is left out.)  Tiles of 4096
+// points take 7 % more at equal figures.
+double mixed_cost(int n, const int *radix, int nstages, int tile)
+{
+    const int T = tile / 16, cnt = tile / n;
+    double c = 0;
+    for (int t = 0, ns = 1; t < nstages; ns *= radix[t++]) {
+        const int R = radix[t], m = n / R, nb = cnt * m, passes = (nb + T - 1) / T;
+        int wave = 0, lanes = 0;
+        for (int g0 = 0; g0 < 64 && g0 < nb; g0 += 16) {
+            int in[16], out[16], k = 0;
+            for (; k < 16 && g0 + k < nb; ++k) {
+                const int g = g0 + k, j = g % m, base = g / m * n;
+                in[k] = base + j;
+                out[k] = base + j / ns * ns * R + j % ns;
+            }
+            wave += half_warp_wavefronts(in, k);
+            if (t < nstages - 1) wave += half_warp_wavefronts(out, k);  // (the last stage stores to the output)
+            lanes += k;
+        }
+        c += 20.0 * passes * R * T + 12.1 * 16.0 * wave / lanes * R * nb + 379.0 * T;
+    }
+    return c / (cnt * (double)n) * (tile == kMixEMax ? 1.07 : 1.0);
+}
+
+struct MixedBest {
+    double cost;
+    int tile, radix[kMixMaxStages];
+};
+
+// All orders of all factorisations of m into `left` radices, after `depth` of them.
+void mixed_search(int n, int m, int left, int *radix, int depth, MixedBest &best)
+{
+    if (left == 0) {
+        if (m != 1) return;
+        for (int tile = 2048; tile <= kMixEMax; tile *= 2) {
+            if (n > tile) continue;
+            const double c = mixed_cost(n, radix, depth, tile);
+            if (best.cost > 0 && c >= best.cost) continue;
+            best.cost = c;
+            best.tile = tile;
+            for (int i = 0; i < depth; ++i) best.radix[i] = radix[i];
+        }
+        return;
+    }
+    for (int r : {16, 15, 14, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2}) {
+        if (m % r || m > r << 4 * (left - 1)) continue;
+        radix[depth] = r;
+        mixed_search(n, m / r, left - 1, radix, depth + 1, best);
+    }
 }
 
 }  // namespace
 
-bool mixed_schedule(int64_t n, int *nstages, int *radix)
+// The schedule of the fewest stages, and the tile, of the least modelled time.
+bool mixed_schedule(int64_t n, int *nstages, int *radix, int *tile)
 {
     if (n < 2 || n > kMixEMax) return false;
     int64_t m = n;
     for (int p : {7, 5, 3, 2})
         while (m % p == 0) m /= p;
     if (m != 1) return false;
-    for (int s = 1; s <= kMixMaxStages; ++s)
-        for (int top = 2; top <= 16; ++top)
-            if (mixed_search(n, top, s, radix, 0)) {
-                // odd radices first
-                for (int i = 1; i < s; ++i)
-                    for (int j = i; j > 0 && (radix[j] & 1) > (radix[j - 1] & 1); --j) {
-                        const int t = radix[j];
-                        radix[j] = radix[j - 1];
-                        radix[j - 1] = t;
-                    }
-                *nstages = s;
-                return true;
-            }
+    for (int s = 1; s <= kMixMaxStages; ++s) {
+        MixedBest best{};
+        mixed_search((int)n, (int)n, s, radix, 0, best);
+        if (best.cost == 0) continue;
+        for (int i = 0; i < s; ++i) radix[i] = best.radix[i];
+        *nstages = s;
+        *tile = best.tile;
+        return true;
+    }
     return false;
 }
 
 cudaError_t launch_mixed(int sign, const MixedArgs &a, cudaStream_t st)
 {
-    if (mix_tile(a.n) == 2048) return sign < 0 ? mixed_t<-1, 2048>(a, st) : mixed_t<1, 2048>(a, st);
+    if (a.tile == 2048) return sign < 0 ? mixed_t<-1, 2048>(a, st) : mixed_t<1, 2048>(a, st);
     return sign < 0 ? mixed_t<-1, 4096>(a, st) : mixed_t<1, 4096>(a, st);
 }
 

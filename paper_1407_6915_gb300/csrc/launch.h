@@ -207,16 +207,16 @@ struct MixedArgs {
     const float2 *tw;   // stage twiddles: stage t at twoff[t], [r-1][k] = w_{ns R}^{k r}, k < ns
     int *err;
     int64_t nseg, ntiles;
-    int n, segs_per_tile, nstages, out_power;
+    int n, tile, segs_per_tile, nstages, out_power;  // tile: points per tile buffer, 2048 or 4096
     int radix[kMixMaxStages], ns[kMixMaxStages], twoff[kMixMaxStages];
     float rm[kMixMaxStages], rns[kMixMaxStages];  // 1 / (n / radix), 1 / ns
     float scale;
 };
 cudaError_t launch_mixed(int sign, const MixedArgs &a, cudaStream_t st);
-// The radix schedule for n (the fewest stages, odd radices first); false if n
-// has a prime factor above 7 or is too long for one tile.
-bool mixed_schedule(int64_t n, int *nstages, int *radix);
-int mixed_segments_per_tile(int64_t n);
+// The radix schedule and the tile for n (the fewest stages; among those the
+// least modelled time); false if n has a prime factor above 7 or is too long
+// for one tile.
+bool mixed_schedule(int64_t n, int *nstages, int *radix, int *tile);
 // Factorisation and tile widths used for n.
 bool fourstep_shape(int log_n, int *log_n1, int *log_n2, int *log_wa, int *log_wb);
 // The four-step twiddle w_n^{j2 k1} is the product of two table entries,

@@ -767,7 +767,7 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
 {
     if (p->path == PATH_MIXED) {
         MixedArgs a{};
-        const int spt = mixed_segments_per_tile(p->n);
+        const int spt = p->mix_tile / (int)p->n;
         a.in = static_cast<const float2 *>(d_in);
         a.out = d_out;
         a.tw = p->twA;
@@ -775,6 +775,7 @@ int exec_plan(fftseg_plan p, const void *d_in, void *d_out, int64_t nseg, cudaSt
         a.nseg = nseg;
         a.ntiles = (nseg + spt - 1) / spt;
         a.n = (int)p->n;
+        a.tile = p->mix_tile;
         a.segs_per_tile = spt;
         a.nstages = p->mix_nstages;
         a.out_power = p->out_kind == FFTSEG_OUT_POWER;
@@ -1518,7 +1519,7 @@ extern "C" {
 // mixed-radix Stockham stages (k_mixed.cu).  The stage twiddles
 // w_{Ns R}^{k r} are evaluated in double on the host and rounded once.
 int create_mixed(fftseg_plan *out, int64_t n, int64_t batch, int direction, int norm, int out_kind,
-                 unsigned flags, const int *radix, int nstages)
+                 unsigned flags, const int *radix, int nstages, int tile)
 {
     fftseg_plan p = new (std::nothrow) fftseg_plan_s();
     if (!p) return set_error(FFTSEG_E_NOMEM, "plan_create: host allocation failed");
@@ -1539,6 +1540,7 @@ int create_mixed(fftseg_plan *out, int64_t n, int64_t batch, int direction, int 
     if (norm == FFTSEG_NORM_BACKWARD) p->scale = direction == FFTSEG_INVERSE ? (float)(1.0 / (double)n) : 1.f;
     else if (norm == FFTSEG_NORM_ORTHO) p->scale = (float)(1.0 / sqrt((double)n));
     p->mix_nstages = nstages;
+    p->mix_tile = tile;
     std::vector<float2> h;
     int64_t ns = 1;
     for (int t = 0; t < nstages; ++t) {
@@ -1595,9 +1597,9 @@ int fftseg_plan_create(fftseg_plan *out, int64_t n, int64_t batch, int direction
     if (!is_pow2(n)) {
         if (precision != FFTSEG_PREC_FP32)
             return set_error(FFTSEG_E_UNSUPPORTED, "plan_create: lengths that are not powers of two are FP32 only");
-        int radix[kMixMaxStages], nst = 0;
-        if (!(flags & FFTSEG_FLAG_BLUESTEIN) && mixed_schedule(n, &nst, radix))
-            return create_mixed(out, n, batch, direction, norm, out_kind, flags, radix, nst);
+        int radix[kMixMaxStages], nst = 0, tile = 0;
+        if (!(flags & FFTSEG_FLAG_BLUESTEIN) && mixed_schedule(n, &nst, radix, &tile))
+            return create_mixed(out, n, batch, direction, norm, out_kind, flags, radix, nst, tile);
         return create_bluestein(out, n, batch, direction, norm, out_kind, flags);
     }
     if (flags & FFTSEG_FLAG_AUTOTUNE) {  // replace the schedule flags by the fastest measured schedule
@@ -1714,7 +1716,7 @@ int fftseg_plan_info(fftseg_plan p, int64_t info[6])
                                               : (p->ring ? (int64_t)p->ring_nr * p->ring_cs * p->n * 8 : 0);
     info[4] = p->blue_q ? p->batch
               : (p->path == PATH_REAL || p->path == PATH_FRAMES || p->path == PATH_BLUESTEIN) ? p->rchunk
-              : p->path == PATH_MIXED ? mixed_segments_per_tile(p->n)
+              : p->path == PATH_MIXED ? p->mix_tile / p->n
               : p->work ? p->work_segs : p->ring_cs;
     info[5] = launches_per_exec(p, p->batch);
     return FFTSEG_OK;

@@ -84,7 +84,7 @@ struct fftseg_plan_s {
     fftseg_plan_s *inner2 = nullptr;
     // lengths 2^a 3^b 5^c 7^d <= 4096 (mixed-radix path): the radix schedule
     // (twA holds the stage twiddles, stage t at mix_twoff[t])
-    int mix_nstages = 0;
+    int mix_nstages = 0, mix_tile = 0;  // (mix_tile: points per tile buffer)
     int mix_radix[16] = {}, mix_twoff[16] = {};
     float2 *bw = nullptr, *bhat = nullptr;
     int64_t bm = 0;
