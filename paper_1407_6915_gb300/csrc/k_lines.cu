@@ -54,6 +54,104 @@ cudaError_t block_t(BlockArgs a, cudaStream_t st)
     return launch_programmatic(k, (unsigned)grid, B::T, B::SMEM, st, a);
 }
 
+// Segments of n = 4, 8 and 16 points: a warp takes 512 points, 16 (whole
+// segments) a lane, and needs no barrier but its own.  The points come in by
+// coalesced 16-byte loads and change to 16 a lane through the warp's own 4 KiB;
+// the bins go back the same way.  Row l (lane l's points) holds 16-byte chunk c
+// at c ^ (l mod 8), |X|^2 rows (64 bytes) at c ^ (l / 2 mod 4): conflict-free on
+// both sides.  Bound by memory: 2^26 points take 183 us (0.88 of the copy rate),
+// as |X|^2 135 us.  (On the tiles of k_block a thread read its points at a stride
+// of a segment, 32 lanes of n = 16 in one bank pair, and stored them so: n = 16
+// 433 us, |X|^2 330; n = 8 307; n = 4 256.  n = 2 stays there: 176 us against
+// 182, |X|^2 122 against 134.)
+constexpr int kShortWarps = 8;
+
+template <int LOG_L, int S>
+__global__ void __launch_bounds__(32 * kShortWarps, 4) k_short(const BlockArgs a)
+{
+    constexpr int L = 1 << LOG_L;
+    static_assert(LOG_L >= 2 && LOG_L <= 4, "whole segments in 16 points");
+    __shared__ float4 sm[kShortWarps * 256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *const X = sm + warp * 256;
+    const int64_t total = a.nseg << LOG_L;
+    grid_launch_dependents();
+    grid_dependency_wait();
+    for (int64_t u = (int64_t)blockIdx.x * kShortWarps + warp; u * 512 < total; u += (int64_t)gridDim.x * kShortWarps) {
+        const int left = (int)(total - u * 512 < 512 ? total - u * 512 : 512);  // points, an even number
+        const float4 *const in = reinterpret_cast<const float4 *>(a.in + u * 512);
+        float4 q[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            q[r] = 2 * (32 * r + lane) < left ? in[32 * r + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncwarp();  // the unit before has been read
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int row = 4 * r + (lane >> 3);
+            X[8 * row + ((lane ^ row) & 7)] = q[r];
+        }
+        __syncwarp();
+        float2 v[16];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float4 x = X[8 * lane + (c ^ (lane & 7))];
+            v[2 * c] = make_float2(x.x, x.y);
+            v[2 * c + 1] = make_float2(x.z, x.w);
+        }
+#pragma unroll
+        for (int g = 0; g < 16; g += L) dft<L, S>(v + g);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) v[c] = cscale(v[c], a.scale);
+        if (a.out_power) {
+            __syncwarp();  // (rows change size)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                X[4 * lane + (c ^ ((lane >> 1) & 3))] = make_float4(power_of(v[4 * c]), power_of(v[4 * c + 1]),
+                                                                    power_of(v[4 * c + 2]), power_of(v[4 * c + 3]));
+            __syncwarp();
+            float *const out = static_cast<float *>(a.out) + u * 512;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int row = 8 * r + (lane >> 2), e = 4 * (32 * r + lane);
+                const float4 x = X[4 * row + ((lane ^ (row >> 1)) & 3)];
+                if (e + 4 <= left) *reinterpret_cast<float4 *>(out + e) = x;
+                else if (e < left) *reinterpret_cast<float2 *>(out + e) = make_float2(x.x, x.y);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c)  // (this lane's own row)
+                X[8 * lane + (c ^ (lane & 7))] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
+            __syncwarp();
+            float4 *const out = reinterpret_cast<float4 *>(static_cast<float2 *>(a.out) + u * 512);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int row = 4 * r + (lane >> 3);
+                const float4 x = X[8 * row + ((lane ^ row) & 7)];
+                if (2 * (32 * r + lane) < left) out[32 * r + lane] = x;
+            }
+        }
+    }
+}
+
+template <int LOG_L, int S>
+cudaError_t short_t(const BlockArgs &a, cudaStream_t st)
+{
+    auto k = k_short<LOG_L, S>;
+    static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
+    int &per_sm = per_sm_dev[current_device_slot()];
+    if (per_sm == 0) {
+        int occ = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 32 * kShortWarps, 0);
+        if (e != cudaSuccess) return e;
+        per_sm = occ > 0 ? occ : 1;
+    }
+    const int64_t ctas = ((a.nseg << LOG_L) + 512 * kShortWarps - 1) / (512 * kShortWarps);
+    if (ctas == 0) return cudaSuccess;
+    int64_t grid = (int64_t)per_sm * sm_count();
+    if (grid > ctas) grid = ctas;
+    return launch_programmatic(k, (unsigned)grid, 32 * kShortWarps, 0, st, a);
+}
+
 template <int LOG_L>
 struct PassShape {
     // up to 16 lines of up to 1024 points (16 KB..128 KB per tile)
@@ -92,6 +190,9 @@ int pass_log_w(int log_l)
 #define FFTSEG_BLOCK_CASE(LL) \
     case LL: return sign < 0 ? block_t<LL, -1>(a, st) : block_t<LL, 1>(a, st);
 
+#define FFTSEG_SHORT_CASE(LL) \
+    case LL: return sign < 0 ? short_t<LL, -1>(a, st) : short_t<LL, 1>(a, st);
+
 cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cudaStream_t st)
 {
     if (prec != PREC_FP32) {  // tensor-core radix-16 stages: n a power of 16
@@ -108,9 +209,9 @@ cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cuda
     }
     switch (log_n) {
         FFTSEG_BLOCK_CASE(1)
-        FFTSEG_BLOCK_CASE(2)
-        FFTSEG_BLOCK_CASE(3)
-        FFTSEG_BLOCK_CASE(4)
+        FFTSEG_SHORT_CASE(2)
+        FFTSEG_SHORT_CASE(3)
+        FFTSEG_SHORT_CASE(4)
         FFTSEG_BLOCK_CASE(5)
         FFTSEG_BLOCK_CASE(6)
         FFTSEG_BLOCK_CASE(7)
