@@ -1,12 +1,12 @@
 // Overlapping segments (frames): frame f of a signal holds samples
 // [f*hop, f*hop + n), multiplied point by point by a real window w[j]
 // (rectangular or periodic Hann, evaluated in double and rounded once).
-// Frames of n <= 4096 points run in one fused pass (k_warp_frames for n = 256,
-// 512 and 1024, else k_block_frames).  Longer
-// frames go in chunks: k_frames copies a chunk of windowed frames into an
-// intermediate that the batched complex plan of n points then transforms; the
-// chunk is sized so that the intermediate stays in L2 between the two passes,
-// and overlapping frames re-read their shared samples from L2.
+// Frames of n <= 4096 points run in one fused pass (k_warp_frames for most of
+// n = 256, 512 and 1024, else k_block_frames).  Longer frames go in chunks:
+// k_frames copies a chunk of windowed frames into an intermediate that the
+// batched complex plan of n points then transforms; the chunk is sized so that
+// the intermediate stays in L2 between the two passes, and overlapping frames
+// re-read their shared samples from L2.
 #include "launch.h"
 #include "programmatic.h"
 
@@ -49,11 +49,16 @@ __global__ void __launch_bounds__(kFrameThreads) k_frames(const FramesArgs a)
 // the first stage gathers its inputs, the n-point forward FFT runs, and the
 // bins are stored from the last stage.  The samples that neighbouring frames
 // share are re-read from L2; each bin crosses HBM once.
+// (frames of 256 side by side: 2^27 points in tiles of 4096 points 342 us, of
+// 2048 355)
+template <int LOG_L>
+constexpr int kFramesLogE = LOG_L == 8 ? 12 : kBlockLogE<LOG_L>;
+
 template <int LOG_L, bool BULK>
-__global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (BlockShape<LOG_L, kBlockLogE<LOG_L>>::PER_SM))
+__global__ void __launch_bounds__((BlockShape<LOG_L, kFramesLogE<LOG_L>>::T), (BlockShape<LOG_L, kFramesLogE<LOG_L>>::PER_SM))
     k_block_frames(const FramesBlockArgs a)
 {
-    using Sh = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
+    using Sh = BlockShape<LOG_L, kFramesLogE<LOG_L>>;
     constexpr int L = 1 << LOG_L, W = 1 << Sh::LOG_W, T = Sh::T, E = Sh::E, V = E / T;
     extern __shared__ __align__(1024) float2 sm[];
     float2 *S = sm;          // staging tiles [2][W][L]
@@ -77,11 +82,13 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (Bl
             const int64_t rows = a.nframes - f0 < W ? a.nframes - f0 : W;
             const float2 *src = a.signal + f0 * a.hop;
             if constexpr (BULK) {
-                if (tid == 0) {
+                static_assert(W <= 32, "a lane per frame");
+                if (tid < 32) {
                     fence_proxy_async();
-                    mbar_expect_tx(&bar[b], (uint32_t)(rows * L * (int64_t)sizeof(float2)));
-                    for (int c = 0; c < rows; ++c)
-                        tma_load_1d(S + b * E + c * L, src + c * a.hop, L * (uint32_t)sizeof(float2), &bar[b]);
+                    if (tid == 0) mbar_expect_tx(&bar[b], (uint32_t)(rows * L * (int64_t)sizeof(float2)));
+                    __syncwarp();
+                    if (tid < rows)
+                        tma_load_1d(S + b * E + tid * L, src + tid * a.hop, L * (uint32_t)sizeof(float2), &bar[b]);
                 }
             } else {
 #pragma unroll
@@ -123,6 +130,7 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kBlockLogE<LOG_L>>::T), (Bl
             if (scale != 1.f) x = make_float2(x.x * scale, x.y * scale);
             const int64_t o = (f0 + c) * L + i;
             if (a.out_power) static_cast<float *>(a.out)[o] = x.x * x.x + x.y * x.y;
+            else if (LOG_L == 8) __stcs(static_cast<float2 *>(a.out) + o, x);  // (333 us, not 342; longer frames 3 % slower)
             else static_cast<float2 *>(a.out)[o] = x;
         });
         __syncthreads();  // S[b] and X read in full before they are rewritten
@@ -225,7 +233,7 @@ cudaError_t warp_frames_t(const FramesBlockArgs &a, cudaStream_t st)
 template <int LOG_L, bool BULK>
 cudaError_t block_frames_launch(FramesBlockArgs a, cudaStream_t st)
 {
-    using B = BlockShape<LOG_L, kBlockLogE<LOG_L>>;
+    using B = BlockShape<LOG_L, kFramesLogE<LOG_L>>;
     constexpr size_t smem = (size_t)(B::SLOTS + 2 * B::E) * sizeof(float2) + 2 * sizeof(uint64_t);
     auto k = k_block_frames<LOG_L, BULK>;
     static int per_sm_dev[kMaxDevices] = {};  // per instantiation and device
@@ -246,21 +254,22 @@ cudaError_t block_frames_launch(FramesBlockArgs a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Frames of 256, 512 and 1024 points a warp at a time.  Others by tiles: bulk
-// copies want 16-byte aligned frames (an even hop on an aligned signal); below
-// 256 points a tile has too many frames for one issuing thread.
+// Frames of 256, 512 and 1024 points a warp at a time where they overlap or go
+// out as |X|^2.  Others by tiles, whose copies ahead keep the memory busier where
+// each sample is read once and a bin is 8 bytes (2^26 points of 1024 at hop 1024
+// 170 us against 180 a warp at a time, of 512 at hop 512 168 and 184, 2^27 of 256
+// at hop 256 333 and 356): bulk copies want 16-byte aligned frames (an even hop on
+// an aligned signal); below 256 points a tile has too many frames for one issuing
+// thread.
 template <int LOG_L>
 cudaError_t block_frames_t(const FramesBlockArgs &a, cudaStream_t st)
 {
-    if constexpr (LOG_L >= 8 && LOG_L <= 10) {
-        return warp_frames_t<(1 << LOG_L) / 32>(a, st);
-    } else {
-        if constexpr (LOG_L > 10) {
-            if ((a.hop & 1) == 0 && (reinterpret_cast<uintptr_t>(a.signal) & 15) == 0)
-                return block_frames_launch<LOG_L, true>(a, st);
-        }
-        return block_frames_launch<LOG_L, false>(a, st);
-    }
+    if constexpr (LOG_L >= 8 && LOG_L <= 10)
+        if (a.hop < (1 << LOG_L) || a.out_power) return warp_frames_t<(1 << LOG_L) / 32>(a, st);
+    if constexpr (LOG_L >= 8)
+        if ((a.hop & 1) == 0 && (reinterpret_cast<uintptr_t>(a.signal) & 15) == 0)
+            return block_frames_launch<LOG_L, true>(a, st);
+    return block_frames_launch<LOG_L, false>(a, st);
 }
 
 }  // namespace
