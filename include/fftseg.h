@@ -86,8 +86,8 @@ enum { FFTSEG_WINDOW_RECT = 0, FFTSEG_WINDOW_HANN = 1 };
    real length.  Runs as a complex FFT of n/2 points on the samples read as
    complex values, plus the split (forward) or join (inverse) of the spectra of
    the even and odd samples: inside the transform's own kernel where it can
-   (forward n <= 2^17; inverse n = 2^14, 2^15 for batches of up to 64 MiB of
-   samples), else as a pass of its own over chunks of at most 512 MiB. */
+   (forward n <= 2^17; inverse n <= 2^13, and n = 2^14, 2^15 for batches of up
+   to 64 MiB of samples), else as a pass of its own over chunks of at most 512 MiB. */
 #define FFTSEG_FLAG_REAL 0x20u
 /* four-step path, FP32, complex output, n = 2^16: the 256 x 256 warp-line
    kernel (16 points per lane, three CTAs per SM) instead of the default
@@ -95,7 +95,7 @@ enum { FFTSEG_WINDOW_RECT = 0, FFTSEG_WINDOW_HANN = 1 };
    default for n = 2^16..2^20) */
 #define FFTSEG_FLAG_FOURSTEP_WARP_LINES 0x40u
 /* four-step path on the CTA-tile kernel (tiles of whole CTAs, the form that
-   also runs |X|^2 output and the tensor-core stages), instead of the
+   also runs the tensor-core stages at n = 2^20 and 2^24), instead of the
    lane-line kernels */
 #define FFTSEG_FLAG_FOURSTEP_TILES 0x80u
 /* test only, for the lane-line kernel: the row tiles of the first segment wait
@@ -106,7 +106,8 @@ enum { FFTSEG_WINDOW_RECT = 0, FFTSEG_WINDOW_HANN = 1 };
    status, not a hang. */
 #define FFTSEG_FLAG_TEST_STALL 0x1000u
 /* lengths that are not powers of two: Bluestein's algorithm even where the
-   mixed-radix path applies (n = 2^a 3^b 5^c 7^d <= 4096) */
+   mixed-radix path applies (n = 2^a 3^b 5^c 7^d <= 4096), and over a power of
+   two of points even where the row kernel applies (n = 2049..12288) */
 #define FFTSEG_FLAG_BLUESTEIN 0x2000u
 
 #define FFTSEG_MAX_LOG2N 24
@@ -121,7 +122,9 @@ typedef struct fftseg_plan_s *fftseg_plan;
  *   n          a power of two, 2 <= n <= 2^24; or any other length 3 <= n <= 2^23
  *              (FP32 only): n = 2^a 3^b 5^c 7^d <= 4096 by mixed-radix stages in
  *              one pass; otherwise by Bluestein's chirp-z identity as a cyclic
- *              convolution over M = 2^ceil(log2(2n - 1)) points: chirp in, M-point
+ *              convolution over M = 2^ceil(log2(2n - 1)) points (n = 2049..12288, without
+ *              schedule flags: the next multiple of 1024, one kernel, no
+ *              workspace): chirp in, M-point
  *              FFT, product with the plan's chirp spectrum, M-point inverse FFT,
  *              chirp out (one launch for M <= 4096, two per chunk for
  *              M = 2^13..2^16, five above; chunks of at most 1 GiB of M-point
@@ -317,7 +320,8 @@ int fftseg_plan_destroy(fftseg_plan p);
 /* Plan facts: info[0] path (0 block, 1 cluster, 2 two-pass, 3 tensor core,
  * 4 persistent four-step, 5 real signal over an inner complex plan,
  * 6 overlapping frames over an inner complex plan, 7 a length that is not a
- * power of two, over two inner plans of M points; info[1] is then M),
+ * power of two, by Bluestein's algorithm over M points; info[1] is then M,
+ * 8 mixed-radix stages, 9 a segment in one SM),
  * info[1] n1, info[2] n2, info[3] workspace bytes, info[4] segments per
  * workspace chunk, info[5] kernel launches per fftseg_exec of a full batch. */
 int fftseg_plan_info(fftseg_plan p, int64_t info[6]);

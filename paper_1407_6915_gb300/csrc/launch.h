@@ -21,7 +21,8 @@ inline int current_device_slot()
 }
 
 // Single-pass segment-major tiles for n = 2^log_n <= 4096 (persistent CTAs,
-// a.ntiles tiles of whole segments; a.ntiles is set by the launcher).  Returns the launch error.
+// a.ntiles tiles of whole segments, set by the launcher; FP32 n = 4, 8, 16: 512
+// points a warp).  Returns the launch error.
 // prec: PREC_FP32, or PREC_FP16 / PREC_BF16 (tensor-core radix-16 stages, n = 16, 256, 4096).
 cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cudaStream_t st);
 int device_sm_count();
@@ -93,7 +94,7 @@ struct FourStepHwArgs;
 cudaError_t launch_fourstep_hw(int sign, const FourStepHwArgs &a, cudaStream_t st);
 // Lane-line persistent four-step kernel for n = 2^16..2^20 (FP32, complex
 // output): lines of 256..1024 points with 32 points per lane, a queue of
-// column and row tiles, loader and retirer warps, swizzled TMA tiles.  prec as
+// column and row tiles, a loader warp and a retirer warp per buffer, swizzled TMA tiles.  prec as
 // for launch_block (tensor-core lines at n = 2^16).
 struct FourStepWlArgs;
 cudaError_t launch_fourstep_wl(int log_n, int sign, int prec, const FourStepWlArgs &a, cudaStream_t st);

@@ -1,5 +1,5 @@
-// Programmatic dependent launch for the single-pass kernels (block,
-// real-signal block and mixed-radix).
+// Programmatic dependent launch for the single-pass kernels (block, short
+// segments, real-signal block, warp frames and mixed-radix).
 #pragma once
 #include <cuda_runtime.h>
 
