@@ -149,7 +149,9 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kFramesLogE<LOG_L>>::T), (B
 // against 223 us for the tiles of k_block_frames, which spend their time between
 // barriers (three stages and two exchanges of the whole CTA); of 512 at hop 256
 // 0.80.  (Each unit's samples prefetched into L2 a unit ahead measured slower,
-// 170 us: the loads of 16 warps keep the memory busy as it is.)
+// 170 us: the loads of 16 warps keep the memory busy as it is.)  The samples are
+// read by plain loads, not __ldg: the kernel before may write them while this
+// one's blocks are resident, and grid_dependency_wait orders plain loads only.
 template <int A>
 __global__ void __launch_bounds__(128, 4) k_warp_frames(const FramesBlockArgs a)
 {
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(128, 4) k_warp_frames(const FramesBlockArgs a)
             const int64_t f = u * G + g;
             const float2 *const x = a.signal + (f < a.nframes ? f : a.nframes - 1) * a.hop + lane;
 #pragma unroll
-            for (int r = 0; r < A; ++r) v[g * A + r] = __ldg(x + 32 * r);
+            for (int r = 0; r < A; ++r) v[g * A + r] = x[32 * r];
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
