@@ -92,6 +92,18 @@ HDEV float2 cscale(float2 a, float s)
 #endif
 }
 
+// a.x * s.x, a.y * s.y
+HDEV float2 cmul_each(float2 a, float2 s)
+{
+#ifdef __CUDA_ARCH__
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(s)));
+    return unpack2(r);
+#else
+    return make_float2(a.x * s.x, a.y * s.y);
+#endif
+}
+
 // a * s + b, s real
 HDEV float2 cfma(float2 a, float s, float2 b)
 {

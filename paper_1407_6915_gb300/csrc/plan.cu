@@ -40,7 +40,7 @@ bool lane_kernels_apply(const fftseg_plan_s *p)
 // Tensor-core precisions at n = 256 x 256: the lane-line kernel with
 // tensor-core lines (wl_tc.cuh) instead of the CTA-tile kernel, whose operands
 // and results all pass through shared memory (1024 segments: 1159 us against
-// 439 us).  Longer ones have lines that are not 16 x 16 points.
+// 451 us).  Longer ones have lines that are not 16 x 16 points.
 bool uses_wl_tc(const fftseg_plan_s *p)
 {
     return p->precision != FFTSEG_PREC_FP32 && p->log_n == 16 &&

@@ -16,10 +16,14 @@
 // b = 2 G + (g >> 2).  So C's two butterflies are one b of two neighbouring
 // lines: a 16-byte store.
 //
-// FP16 operands are scaled into range by a power of two taken from the group's
-// largest component (one warp reduction per group, scaled back exactly).
-// Elements within 2^-15 of that maximum keep all 22 bits of the split; for
-// smaller ones the error stays below 2^-38 of the maximum.
+// FP16 operands are scaled into range by a power of two taken from the
+// butterfly's largest component and scaled back exactly, as dft16_tc does.  The
+// four lanes of a butterfly find its exponent by two shuffles, and two more bring
+// a lane those of its two output butterflies: 451 us for the 1024 segments below.
+// (One maximum for the eight butterflies of a group, by a warp reduction, took
+// 432 but left a quiet line beside a loud one with fewer bits, down to an error of
+// 1.7e-3 at 2^-30 of its neighbour.  That maximum where the group is even and
+// the shuffles else, 496; four groups' exponents in the bytes of one word, 470.)
 //
 // Tile rows: element (hi, lo) of a line, hi, lo < 16, is in row 16 hi + lo, its
 // 16-byte chunk at (column / 2) ^ (lo & 7) ^ X(hi).  Input tiles hold point
@@ -31,7 +35,7 @@
 // exchange puts bin k of butterfly b at (k, b ^ 2 (k & 1)).  Every access is
 // conflict-free but the row tiles' staged output (two-way).
 //
-// 1024 segments of 65536 points, FP16 hi+lo: 432 us (BF16: 375 us) against
+// 1024 segments of 65536 points, FP16 hi+lo: 451 us (BF16: 376 us) against
 // 1159 us on the CTA-tile kernel, whose operands, hi and lo, and results all
 // pass through shared memory once more per stage.  Tensor pipe 37 % active,
 // shared-memory pipe 35 %, issue 35 %: bound by latency, with two compute warps
@@ -67,9 +71,9 @@ struct WlTcF {
 
 // Eight butterflies: d[mt] = (re, re', im, im') of bin g + 8 mt of butterflies
 // 2 t and 2 t + 1 from this lane's points x[i] = t + 4 i of butterfly g, scaled
-// by sc (FP16) and back by inv.
+// by sc (FP16) and the two back by inv.
 template <int PREC>
-FDEV void wl_tc_group(float (&d)[2][4], const float2 (&x)[4], float sc, float inv, const WlTcF &F)
+FDEV void wl_tc_group(float (&d)[2][4], const float2 (&x)[4], float sc, float2 inv, const WlTcF &F)
 {
     uint32_t xh[4], xl[4];
 #pragma unroll
@@ -94,7 +98,7 @@ FDEV void wl_tc_group(float (&d)[2][4], const float2 (&x)[4], float sc, float in
         if constexpr (PREC == PREC_FP16) {
 #pragma unroll
             for (int i = 0; i < 4; i += 2) {
-                const float2 y = cscale(make_float2(d[mt][i], d[mt][i + 1]), inv);
+                const float2 y = cmul_each(make_float2(d[mt][i], d[mt][i + 1]), inv);
                 d[mt][i] = y.x;
                 d[mt][i + 1] = y.y;
             }
@@ -114,38 +118,45 @@ FDEV void wl_tc_line(float (&d)[8][2][4], char *Pc, uint32_t pb, int w, int g, i
     const uint32_t X = ROWS ? (uint32_t)qx : 0u;
     const uint32_t lc = (uint32_t)(w + 4 * ((g >> 1) & 1)) ^ X, rd = pb + 2048 * (g >> 2) + 8 * (g & 1);
     const uint32_t lw = (uint32_t)(w + 4 * (t & 1)) ^ X;
-    // four groups' points and scales before their products: one wait for the
-    // tile and the warp reductions instead of four (FP16 439 -> 432 us; all
-    // eight groups 440, two 440)
+    // GB groups' points and scales before their products: one wait for the tile
+    // and the shuffles instead of GB (FP16: 451 us with two, 470 with four, 464
+    // with eight; BF16, which has no scales: 376 with four)
+    constexpr int GB = PREC == PREC_FP16 ? 2 : 4;
     auto pass = [&](uint32_t t0) {
         const uint32_t base = rd + 128 * t0 + 16 * (lc ^ t0);
 #pragma unroll
-        for (int G0 = 0; G0 < 8; G0 += 4) {
-            float2 x[4][4];
-            uint32_t top[4];
+        for (int G0 = 0; G0 < 8; G0 += GB) {
+            float2 x[GB][4];
+            [[maybe_unused]] uint32_t e[GB];  // biased exponent of the butterfly's largest component, in place
 #pragma unroll
-            for (int G = 0; G < 4; ++G)
+            for (int G = 0; G < GB; ++G)
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
                     x[G][i] = *reinterpret_cast<const float2 *>(
                         Pc + ((base ^ KX(4 * i) ^ (ROWS && G0 + G >= 4 ? 64u : 0u)) + 4096u * (G0 + G)));
             if constexpr (PREC == PREC_FP16) {
+                float m[GB];
 #pragma unroll
-                for (int G = 0; G < 4; ++G) {
-                    float mx = 0.f;
+                for (int G = 0; G < GB; ++G) {
+                    m[G] = 0x1p-100f;  // (both scales are normal)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) mx = fmaxf(mx, fmaxf(fabsf(x[G][i].x), fabsf(x[G][i].y)));
-                    top[G] = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+                    for (int i = 0; i < 4; ++i) m[G] = fmaxf(m[G], fmaxf(fabsf(x[G][i].x), fabsf(x[G][i].y)));
                 }
+#pragma unroll
+                for (int G = 0; G < GB; ++G) m[G] = fmaxf(m[G], __shfl_xor_sync(0xffffffffu, m[G], 1));
+#pragma unroll
+                for (int G = 0; G < GB; ++G)
+                    e[G] = __float_as_uint(fmaxf(m[G], __shfl_xor_sync(0xffffffffu, m[G], 2))) & 0x7f800000u;
             }
 #pragma unroll
-            for (int G = 0; G < 4; ++G) {
-                float sc = 1.f, inv = 1.f;
-                if constexpr (PREC == PREC_FP16) {
-                    int e = (int)(top[G] >> 23) - 127;  // floor(log2) of a normal maximum
-                    e = e < -100 ? -100 : (e > 100 ? 100 : e);
-                    sc = __uint_as_float((uint32_t)(127 + 13 - e) << 23);
-                    inv = __uint_as_float((uint32_t)(127 - 13 + e) << 23);
+            for (int G = 0; G < GB; ++G) {
+                float sc = 1.f;
+                float2 inv = make_float2(1.f, 1.f);
+                if constexpr (PREC == PREC_FP16) {  // 2^(13 - e), and 2^(e - 13) of the output butterflies
+                    sc = __uint_as_float((267u << 23) - e[G]);
+                    const uint32_t u = e[G] - (13u << 23);
+                    inv = make_float2(__uint_as_float(__shfl_sync(0xffffffffu, u, 8 * t)),
+                                      __uint_as_float(__shfl_sync(0xffffffffu, u, 8 * t + 4)));
                 }
                 wl_tc_group<PREC>(d[G0 + G], x[G], sc, inv, F);
             }
