@@ -572,8 +572,8 @@ __global__ void __launch_bounds__(FourStepWlShape<LOG_N1, LOG_N2, LOG_E, NB, MIN
                 float d[8][2][4];
                 const uint32_t pb = tb + (uint32_t)(tp * PA::PANEL_BYTES);
                 const int tile = item[4 * bb + 2];
-                if (kind == KIND_A) wl_tc_line<S, PREC, false>(d, Pc, pb, tw, tg, tt, 0, tcf, tctw);
-                else wl_tc_line<S, PREC, true>(d, Pc, pb, tw, tg, tt, (2 * tile + tp) & 3, tcf, tctw);
+                if (kind == KIND_A) wl_tc_line<S, PREC, false>(d, Pc, pb, tw, tg, tt, 0, tcf, tctw, a.err);
+                else wl_tc_line<S, PREC, true>(d, Pc, pb, tw, tg, tt, (2 * tile + tp) & 3, tcf, tctw, a.err);
                 const int c0 = 2 * tw + 8 * (tt & 1);  // the lane's first line in its panel
                 if (kind == KIND_A) {
                     // times w_n^{j2 k1} (two factors, scale folded in), staged as [q][column][16 k]

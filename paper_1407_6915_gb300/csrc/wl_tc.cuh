@@ -112,8 +112,13 @@ FDEV void wl_tc_group(float (&d)[2][4], const float2 (&x)[4], float sc, float2 i
 // lines 2 w + 8 (t & 1) and the next.
 template <int S, int PREC, bool ROWS>
 FDEV void wl_tc_line(float (&d)[8][2][4], char *Pc, uint32_t pb, int w, int g, int t, int qx, const WlTcF &F,
-                     const float2 (&tw)[8][2])
+                     const float2 (&tw)[8][2], [[maybe_unused]] int *err)
 {
+    // (self-checking build: every slot of size bytes within the panel, aligned)
+    auto at = [&](uint32_t off, [[maybe_unused]] uint32_t size) {
+        if (!FFTSEG_CHECK(off - pb <= 32768 - size && off % size == 0, err)) off = pb;
+        return Pc + off;
+    };
     auto KX = [](uint32_t x) { return 128 * x + 16 * (x & 7); };  // row and chunk bits of lo
     const uint32_t X = ROWS ? (uint32_t)qx : 0u;
     const uint32_t lc = (uint32_t)(w + 4 * ((g >> 1) & 1)) ^ X, rd = pb + 2048 * (g >> 2) + 8 * (g & 1);
@@ -133,7 +138,7 @@ FDEV void wl_tc_line(float (&d)[8][2][4], char *Pc, uint32_t pb, int w, int g, i
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
                     x[G][i] = *reinterpret_cast<const float2 *>(
-                        Pc + ((base ^ KX(4 * i) ^ (ROWS && G0 + G >= 4 ? 64u : 0u)) + 4096u * (G0 + G)));
+                        at((base ^ KX(4 * i) ^ (ROWS && G0 + G >= 4 ? 64u : 0u)) + 4096u * (G0 + G), 8));
             if constexpr (PREC == PREC_FP16) {
                 float m[GB];
 #pragma unroll
@@ -172,7 +177,7 @@ FDEV void wl_tc_line(float (&d)[8][2][4], char *Pc, uint32_t pb, int w, int g, i
         for (int mt = 0; mt < 2; ++mt) {
             const float2 a = twmul<S>(make_float2(d[G][mt][0], d[G][mt][2]), tw[G][mt]);
             const float2 b = twmul<S>(make_float2(d[G][mt][1], d[G][mt][3]), tw[G][mt]);
-            *reinterpret_cast<float4 *>(Pc + ((wb ^ KX(2 * G) ^ (ROWS && mt ? 64u : 0u)) + 16384u * mt)) =
+            *reinterpret_cast<float4 *>(at((wb ^ KX(2 * G) ^ (ROWS && mt ? 64u : 0u)) + 16384u * mt, 16)) =
                 make_float4(a.x, a.y, b.x, b.y);
         }
     __syncwarp();
