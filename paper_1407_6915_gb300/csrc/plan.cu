@@ -1435,8 +1435,9 @@ int create_bluestein(fftseg_plan *out, int64_t n, int64_t batch, int direction, 
     else if (norm == FFTSEG_NORM_ORTHO) p->scale = (float)(1.0 / sqrt((double)n));
     // n = 2049..12288: rows of q * 1024 points in one SM each, in one launch
     // (an asked-for schedule, and FFTSEG_FLAG_BLUESTEIN, which asks for
-    // power-of-two rows, keep the passes over rows of M points)
-    const int q = flags & (kPathFlags | FFTSEG_FLAG_AUTOTUNE | FFTSEG_FLAG_BLUESTEIN) ? 0 : blue_row_q(n);
+    // power-of-two rows, keep the passes over rows of M points; FFTSEG_FLAG_AUTOTUNE
+    // asks for the fastest, which is this one at every length and batch measured)
+    const int q = flags & (kPathFlags | FFTSEG_FLAG_BLUESTEIN) ? 0 : blue_row_q(n);
     if (q) {
         const int64_t m = (int64_t)q * 1024;
         std::vector<float2> w, h;
