@@ -1,5 +1,6 @@
 // Programmatic dependent launch for the single-pass kernels (block, short
-// segments, real-signal block, warp frames and mixed-radix).
+// segments, real-signal block, warp frames, mixed-radix, and small batches of
+// the kernels with a segment or a Bluestein row per SM).
 #pragma once
 #include <cuda_runtime.h>
 

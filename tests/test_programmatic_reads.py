@@ -35,7 +35,7 @@ def kernels():
 
 def test_programmatic_kernels_read_only_tables_through_ldg():
     found = {name: body for name, body in kernels() if "grid_dependency_wait" in body}
-    assert {"k_block", "k_short", "k_mixed", "k_block_r2c", "k_block_c2r", "k_warp_frames"} <= set(found)
+    assert {"k_block", "k_short", "k_mixed", "k_block_r2c", "k_block_c2r", "k_warp_frames", "k_one_sm"} <= set(found)
     for name, body in found.items():
         for arg in re.findall(r"__ldg\(\s*&?([\w.]+)", body):
             assert arg in TABLES, (name, arg)
@@ -71,5 +71,38 @@ def test_frames_of_a_signal_rewritten_in_place(n, between):
 
     ref = chain(True)
     for _ in range(20):
+        for got, want in zip(chain(False), ref):
+            assert torch.equal(got, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,B", [(1 << 14, 1), (1 << 14, 40), (1 << 14, 90)])
+def test_chains_of_small_batches(n, B):
+    # every call reads what the call before wrote, a few segments and more than
+    # are launched programmatically: the same bits as with a wait between calls
+    torch = pytest.importorskip("torch")
+    import paper_1407_6915_gb300 as fs
+
+    a0 = torch.from_numpy(siggen.uniform(3700 + n, B * n).reshape(B, n)).cuda()
+    plans = [fs.Plan(n, B, d, fs.NORM_ORTHO) for d in (fs.FORWARD, fs.INVERSE)]
+    power = fs.Plan(n, B, fs.FORWARD, fs.NORM_ORTHO, out_kind=fs.OUT_POWER)
+
+    def chain(sync):
+        a, b = a0.clone(), torch.empty_like(a0)
+        p = [torch.empty((B, n), dtype=torch.float32, device="cuda") for _ in range(4)]
+        torch.cuda.synchronize()
+        for i in range(4):
+            for plan, src, dst in ((plans[0], a, b), (power, b, p[i]), (plans[1], b, a), (plans[0], a, b),
+                                   (plans[0], b, a)):
+                plan.exec(src, out=dst)
+                if sync:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        for plan in plans + [power]:
+            plan.check()
+        return [a, b] + p
+
+    ref = chain(True)
+    for _ in range(10):
         for got, want in zip(chain(False), ref):
             assert torch.equal(got, want)
