@@ -26,6 +26,7 @@
 
 #include "launch.h"
 #include "plan.h"
+#include "programmatic.h"
 
 namespace fftseg {
 
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(BlueRowShape<Q>::T, BlueRowShape<Q>::PER_SM) k
     extern __shared__ float2 sm[];
     float2 *const TW = sm + Sh::M;  // w_1024^{j2 t} at [t][j2]
     const int tid = threadIdx.x;
+    grid_launch_dependents();
     for (int e = tid; e < kRow; e += T) TW[e] = __ldg(a.tw2 + e);
     const int n = a.n;
     // w_M^{j r} from [b-1][j], b = 1..3, then [a-1][j] for w_M^{4 a j}
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(BlueRowShape<Q>::T, BlueRowShape<Q>::PER_SM) k
 #pragma unroll
         for (int r = 1; r < Q; ++r) w[r] = r < 4 ? wb[r] : (r & 3) ? cmul(wa[r >> 2], wb[r & 3]) : wa[r >> 2];
     };
+    grid_dependency_wait();
     __syncthreads();
     for (int64_t row = blockIdx.x; row < a.nseg; row += gridDim.x) {
         const float2 *const x = a.x + row * n;
@@ -87,7 +90,7 @@ __global__ void __launch_bounds__(BlueRowShape<Q>::T, BlueRowShape<Q>::PER_SM) k
             for (int r = 0; r < H; ++r) {
                 v[r] = c[r] = make_float2(0.f, 0.f);
                 if (j + kRow * r < n) {
-                    v[r] = __ldg(x + j + kRow * r);
+                    v[r] = x[j + kRow * r];
                     c[r] = __ldg(a.w + j + kRow * r);
                 }
             }
@@ -206,6 +209,9 @@ cudaError_t blue_row_t(const BlueRowArgs &a, cudaStream_t st)
     int64_t grid = (int64_t)per_sm * device_sm_count();
     if (grid > a.nseg) grid = a.nseg;
     if (grid < 1) return cudaSuccess;
+    // a few rows: as k_one_sm (calls of 8 rows of 10007, one after the other: 20.7 ->
+    // 18.0 us; the two cluster passes, which spread a row over eight SMs, 18.9)
+    if (a.nseg <= device_sm_count() / 2) return launch_programmatic(k, (unsigned)grid, Sh::T, Sh::SMEM, st, a);
     k<<<(unsigned)grid, Sh::T, Sh::SMEM, st>>>(a);
     return cudaGetLastError();
 }

@@ -13,7 +13,7 @@ import pytest
 import siggen
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1407_6915_gb300", "csrc")
-TABLES = {"a.tw", "a.twL", "a.twW", "a.window", "tw"}  # plan tables, complete before a plan is returned
+TABLES = {"a.tw", "a.tw1", "a.tw2", "a.bhat", "a.w", "a.twL", "a.twW", "a.window", "tw"}  # plan tables, complete before a plan is returned
 
 
 def kernels():
@@ -35,7 +35,8 @@ def kernels():
 
 def test_programmatic_kernels_read_only_tables_through_ldg():
     found = {name: body for name, body in kernels() if "grid_dependency_wait" in body}
-    assert {"k_block", "k_short", "k_mixed", "k_block_r2c", "k_block_c2r", "k_warp_frames", "k_one_sm"} <= set(found)
+    assert {"k_block", "k_short", "k_mixed", "k_block_r2c", "k_block_c2r", "k_warp_frames", "k_one_sm",
+            "k_blue_row"} <= set(found)
     for name, body in found.items():
         for arg in re.findall(r"__ldg\(\s*&?([\w.]+)", body):
             assert arg in TABLES, (name, arg)
@@ -76,7 +77,8 @@ def test_frames_of_a_signal_rewritten_in_place(n, between):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,B", [(1 << 14, 1), (1 << 14, 40), (1 << 14, 90)])
+@pytest.mark.parametrize("n,B", [(1 << 14, 1), (1 << 14, 40), (1 << 14, 90), (10007, 1), (10007, 40), (2049, 90),
+                                 (12281, 9)])
 def test_chains_of_small_batches(n, B):
     # every call reads what the call before wrote, a few segments and more than
     # are launched programmatically: the same bits as with a wait between calls
