@@ -72,12 +72,12 @@ __global__ void __launch_bounds__(32 * kShortWarps, 4) k_short(const BlockArgs a
     constexpr int L = 1 << LOG_L;
     static_assert(LOG_L >= 2 && LOG_L <= 4, "whole segments in 16 points");
     __shared__ float4 sm[kShortWarps * 256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     float4 *const X = sm + warp * 256;
     const int64_t total = a.nseg << LOG_L;
     grid_launch_dependents();
     grid_dependency_wait();
-    for (int64_t u = (int64_t)blockIdx.x * kShortWarps + warp; u * 512 < total; u += (int64_t)gridDim.x * kShortWarps) {
+    for (int64_t u = (int64_t)blockIdx.x * warps + warp; u * 512 < total; u += (int64_t)gridDim.x * warps) {
         const int left = (int)(total - u * 512 < 512 ? total - u * 512 : 512);  // points, an even number
         const float4 *const in = reinterpret_cast<const float4 *>(a.in + u * 512);
         float4 q[8];
@@ -145,11 +145,16 @@ cudaError_t short_t(const BlockArgs &a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         per_sm = occ > 0 ? occ : 1;
     }
-    const int64_t ctas = ((a.nseg << LOG_L) + 512 * kShortWarps - 1) / (512 * kShortWarps);
-    if (ctas == 0) return cudaSuccess;
+    // A small batch is spread over the SMs, in smaller CTAs (2^14 points of n = 4,
+    // 32 warps: in 4 CTAs 2.07 us, in 32 1.37, on the tiles of k_block 1.48)
+    const int64_t units = ((a.nseg << LOG_L) + 511) / 512;
+    if (units == 0) return cudaSuccess;
+    int64_t warps = (units + sm_count() - 1) / sm_count();
+    if (warps > kShortWarps) warps = kShortWarps;
+    const int64_t ctas = (units + warps - 1) / warps;
     int64_t grid = (int64_t)per_sm * sm_count();
     if (grid > ctas) grid = ctas;
-    return launch_programmatic(k, (unsigned)grid, 32 * kShortWarps, 0, st, a);
+    return launch_programmatic(k, (unsigned)grid, 32 * (unsigned)warps, 0, st, a);
 }
 
 template <int LOG_L>
