@@ -214,7 +214,9 @@ cudaError_t launch_block(int log_n, int sign, int prec, const BlockArgs &a, cuda
     }
     switch (log_n) {
         FFTSEG_BLOCK_CASE(1)
-        FFTSEG_SHORT_CASE(2)
+        case 2:  // |X|^2: 2^20 points 2.7 us on the tiles, 3.7 a warp at a time (2^25: 63 and 65)
+            if (a.out_power) return sign < 0 ? block_t<2, -1>(a, st) : block_t<2, 1>(a, st);
+            return sign < 0 ? short_t<2, -1>(a, st) : short_t<2, 1>(a, st);
         FFTSEG_SHORT_CASE(3)
         FFTSEG_SHORT_CASE(4)
         FFTSEG_BLOCK_CASE(5)
