@@ -8,11 +8,11 @@ namespace fftseg {
 namespace {
 
 template <int LOG_N1, int LOG_N2, int LOG_C, int S, bool RF = false, bool RI = false, bool BL = false,
-          bool BF = false>
+          bool BF = false, int MINB = ClusterShape<LOG_N1, LOG_N2, LOG_C>::MINB>
 cudaError_t cluster_t(const ClusterArgs &a, cudaStream_t st)
 {
     using Sh = ClusterShape<LOG_N1, LOG_N2, LOG_C>;
-    auto k = k_cluster<LOG_N1, LOG_N2, LOG_C, S, RF, RI, BL, BF>;
+    auto k = k_cluster<LOG_N1, LOG_N2, LOG_C, S, RF, RI, BL, BF, MINB>;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -107,8 +107,18 @@ cudaError_t launch_cluster_c2r(int log_n, int log_c, const ClusterArgs &a, cudaS
     if (!cluster_shape(log_n, log_c, &l1, &l2, &lc)) return cudaErrorInvalidValue;
     switch (log_n) {
         // (n/2 = 2^13 and 2^14: larger inverse plans are faster chunked)
-        case 13: return cluster_t<6, 7, 1, 1, false, true>(a, st);
-        case 14: return cluster_t<7, 7, 2, 1, false, true>(a, st);
+        // Registers for two CTAs per SM, not three (80 a thread spill where a point
+        // is joined from two bins and a factor): n/2 = 2^14, 37 segments 9.6 -> 8.6
+        // us, 512 60.9 -> 54.2, but not where three take all segments at once and
+        // two do not (100: 13.4 -> 14.1).  At 2^13 only while two take all at once:
+        // 8 segments 7.2 -> 6.7 us, 100 10.1 -> 9.6, but 200 13.1 -> 14.6.
+        case 13:
+            if (a.nseg <= device_sm_count()) return cluster_t<6, 7, 1, 1, false, true, false, false, 2>(a, st);
+            return cluster_t<6, 7, 1, 1, false, true>(a, st);
+        case 14:
+            if (4 * a.nseg > 2 * device_sm_count() && 4 * a.nseg <= 3 * device_sm_count())
+                return cluster_t<7, 7, 2, 1, false, true>(a, st);
+            return cluster_t<7, 7, 2, 1, false, true, false, false, 2>(a, st);
         default: return cudaErrorInvalidValue;
     }
 }

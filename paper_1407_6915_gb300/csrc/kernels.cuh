@@ -509,8 +509,8 @@ FDEV void rf_place(int k1, int &d, int &c)
 // BF (Bluestein rows, S = -1): the forward transform of the chirped row,
 // read from the n input samples directly (zero past n, no slab copy).
 template <int LOG_N1, int LOG_N2, int LOG_C, int S, bool RF = false, bool RI = false, bool BL = false,
-          bool BF = false>
-__global__ void __launch_bounds__(ClusterShape<LOG_N1, LOG_N2, LOG_C>::T, ClusterShape<LOG_N1, LOG_N2, LOG_C>::MINB)
+          bool BF = false, int MINB = ClusterShape<LOG_N1, LOG_N2, LOG_C>::MINB>
+__global__ void __launch_bounds__(ClusterShape<LOG_N1, LOG_N2, LOG_C>::T, MINB)
     k_cluster(const __grid_constant__ ClusterArgs a)
 {
     constexpr bool DIRECT = RI || BF;  // the column pass reads global memory itself (no slab copy)
