@@ -534,7 +534,6 @@ HDEV void dft(float2 *v)
     else if constexpr (R == 14) dft_coprime<2, 7, S>(v);
     else if constexpr (R == 15) dft_coprime<5, 3, S>(v);
     else if constexpr (R == 18) dft_coprime<2, 9, S>(v);
-    else if constexpr (R == 20) dft_coprime<4, 5, S>(v);
     else if constexpr (R == 24) dft_coprime<8, 3, S>(v);
     else if constexpr (R == 3 || R == 5 || R == 7) dft_odd<R, S>(v);
     else if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);

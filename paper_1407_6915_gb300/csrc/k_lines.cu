@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(32 * kShortWarps, 4) k_short(const BlockArgs a
     grid_launch_dependents();
     grid_dependency_wait();
     for (int64_t u = (int64_t)blockIdx.x * warps + warp; u * 512 < total; u += (int64_t)gridDim.x * warps) {
-        const int left = (int)(total - u * 512 < 512 ? total - u * 512 : 512);  // points, an even number
+        const int left = (int)(total - u * 512 < 512 ? total - u * 512 : 512);  // points, a multiple of 4
         const float4 *const in = reinterpret_cast<const float4 *>(a.in + u * 512);
         float4 q[8];
 #pragma unroll
@@ -114,8 +114,7 @@ __global__ void __launch_bounds__(32 * kShortWarps, 4) k_short(const BlockArgs a
             for (int r = 0; r < 4; ++r) {
                 const int row = 8 * r + (lane >> 2), e = 4 * (32 * r + lane);
                 const float4 x = X[4 * row + ((lane ^ (row >> 1)) & 3)];
-                if (e + 4 <= left) *reinterpret_cast<float4 *>(out + e) = x;
-                else if (e < left) *reinterpret_cast<float2 *>(out + e) = make_float2(x.x, x.y);
+                if (e < left) *reinterpret_cast<float4 *>(out + e) = x;
             }
         } else {
 #pragma unroll
