@@ -123,12 +123,12 @@ typedef struct fftseg_plan_s *fftseg_plan;
  *              (FP32 only): n = 2^a 3^b 5^c 7^d <= 4096 by mixed-radix stages in
  *              one pass; otherwise by Bluestein's chirp-z identity as a cyclic
  *              convolution over M = 2^ceil(log2(2n - 1)) points (n = 2049..12288, without
- *              schedule flags: the next multiple of 1024, one kernel, no
- *              workspace): chirp in, M-point
- *              FFT, product with the plan's chirp spectrum, M-point inverse FFT,
- *              chirp out (one launch for M <= 4096, two per chunk for
- *              M = 2^13..2^16, five above; chunks of at most 1 GiB of M-point
- *              rows; out of place only); else FFTSEG_E_UNSUPPORTED
+ *              schedule flags: M = 1024 q for the smallest q of 5..10, 12, 14,
+ *              15, 16, 18, 20, 24 with M >= 2n - 1, one kernel, no workspace):
+ *              chirp in, M-point FFT, product with the plan's chirp spectrum,
+ *              M-point inverse FFT, chirp out (one launch for M <= 4096, two per
+ *              chunk for M = 2^13..2^16, five above; chunks of at most 1 GiB of
+ *              M-point rows; out of place only); else FFTSEG_E_UNSUPPORTED
  *   batch      >= 1: the most segments one fftseg_exec call processes
  *   direction  FFTSEG_FORWARD or FFTSEG_INVERSE
  *   norm       FFTSEG_NORM_*

@@ -11,8 +11,8 @@
 //        1024 r + 32 t + u; times B there (stored in that order); radix 32 back
 //   S2', S1'  the inverses; the first n points times scale w[m] to the output
 // A point crosses shared memory eight times (8 bytes each), with one barrier
-// per stage, and device memory once each way; M exceeds 2 n - 1 by less than
-// 2048, not by up to a factor of two.  n = 10007 (M = 20480), 2501 rows: 292 us,
+// per stage, and device memory once each way; M exceeds 2 n - 1 by at most 4095
+// (between the built Q = 20 and 24; 2047 below), not by up to a factor of two.  n = 10007 (M = 20480), 2501 rows: 292 us,
 // against 806 us for the two cluster-kernel passes over rows of 32768 points,
 // whose exchange crosses SMs twice (n = 4099, 6000 rows: 299 against 868 us).
 // What bounds it is the chain of stages with 16 warps per SM: issue slots 46 %

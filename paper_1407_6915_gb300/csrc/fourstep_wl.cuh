@@ -65,7 +65,7 @@ struct FourStepWlArgs {
     float2 *ring;        // nr*cs segments, [slot*cs + sl][k1 / PW_B][j2][k1 mod PW_B]
     const float2 *twA;   // stage-2 twiddles of an N1-point line: [r-1][b] = w_{N1}^{b r}, r < P1, b < 32
     const float2 *twB;   // the same for N2
-    const float2 *w4t;   // per column tile ct, columns by pair and half (WlPass::pair_of, c mod 2 fastest):
+    const float2 *w4t;   // per column tile ct, columns by pair and half (WlPass::line_of, the half fastest):
                          // [W_A/2][P1][2] w_n^{j2 j}, then [32][W_A/2][2] scale * w_n^{j2 P1 m}
     int *ctr;            // [0] queue head, [1 + s] column tiles of s done, [1 + nc*cs + s] row tiles of s done
     int *err;

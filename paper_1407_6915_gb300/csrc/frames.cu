@@ -40,11 +40,11 @@ __global__ void __launch_bounds__(kFrameThreads) k_frames(const FramesArgs a)
     *reinterpret_cast<float4 *>(dst) = make_float4(x0.x * w0, x0.y * w0, x1.x * w1, x1.y * w1);
 }
 
-// Frames of n <= 4096 points in one pass: a CTA takes tiles of W = 4096 / n
-// frames (the block kernel's tile shape).  The samples of the next tile are
-// copied asynchronously into one of two staging tiles while the current tile
-// is transformed: with BULK (16-byte aligned frames, n >= 2048) one thread
-// issues a bulk copy per frame, completed on an mbarrier; otherwise every
+// Frames of n <= 4096 points in one pass: a CTA takes tiles of whole frames,
+// 2048 points (4096 at n = 256 and 4096; 256 frames below n = 16).  The samples
+// of the next tile are copied asynchronously into one of two staging tiles while
+// the current tile is transformed: with BULK (16-byte aligned frames, n >= 256) a
+// lane per frame issues its bulk copy, completed on an mbarrier; otherwise every
 // thread issues 8-byte cp.async copies (any hop).  The window is applied as
 // the first stage gathers its inputs, the n-point forward FFT runs, and the
 // bins are stored from the last stage.  The samples that neighbouring frames

@@ -1,5 +1,5 @@
 // Instantiations and launcher of the lane-line persistent four-step kernel
-// (n = 2^16 .. 2^20, FP32, complex output).
+// (n = 2^16 .. 2^20, FP32, complex or |X|^2 output; tensor-core lines at 2^16).
 #include "fourstep_wl.cuh"
 #include "launch.h"
 
@@ -8,7 +8,7 @@ namespace fftseg {
 namespace {
 
 // 8192-point tiles, three buffers, one CTA per SM (eight compute warps of
-// 32 points per lane, a loader warp and a retirer warp).  Measured on GB300:
+// 32 points per lane, a loader warp and a retirer warp per buffer).  Measured on GB300:
 // two buffers were 5-9 % slower.
 // (4096-point tiles at two CTAs per SM measured no faster at 2^16 and
 // 4-27 % slower at 2^17..2^20.)

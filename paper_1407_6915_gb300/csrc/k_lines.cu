@@ -24,11 +24,15 @@ int sm_count()
 template <int LOG_L, int S, int PREC = PREC_FP32, int LOG_E = 12>
 cudaError_t block_t(BlockArgs a, cudaStream_t st)
 {
-    // Up to 2^22 points (32 MiB) in tiles of 2048 points: a launch is a few rounds
-    // of the grid then, and twice as many tiles leave less of the last round idle
-    // (1024 points a segment, us: 2^20 points 5.02 -> 4.59, 2^21 7.91 -> 7.40, 2^22
-    // 13.77 -> 13.35; 2^23 equal, above up to 5 % slower).  The same arithmetic on
-    // every segment, so the same bits.
+    // Up to 2^22 points (32 MiB) in tiles of 2048 points: a launch is at most a few
+    // rounds of the grid then (as many with either tile, the CTAs per SM double
+    // with the tiles), and tiles half as large are in sooner and out sooner, at
+    // the start and the end.  Replayed from a graph over rotating buffers, us with
+    // tiles of 4096 -> 2048 points: n = 1024, 2^18 points 3.63 -> 2.98, 2^20 5.12 ->
+    // 4.61, 2^22 13.53 -> 12.83; n = 32 3.94 -> 3.21, 5.60 -> 5.29, 15.4 -> 14.9;
+    // n = 2048 3.63 -> 2.97, 5.17 -> 4.78, 14.1 -> 13.3; the lengths between and
+    // |X|^2 alike.  From 2^23 points on equal, above up to 5 % slower.  The same
+    // arithmetic on every segment, so the same bits.
     if constexpr (PREC == PREC_FP32 && LOG_E == 12 && kBlockLogE<LOG_L> == 11) {
         if (a.nseg <= (int64_t(1) << 22) >> LOG_L) return block_t<LOG_L, S, PREC, 11>(a, st);
     }
@@ -59,10 +63,11 @@ cudaError_t block_t(BlockArgs a, cudaStream_t st)
 // coalesced 16-byte loads and change to 16 a lane through the warp's own 4 KiB;
 // the bins go back the same way.  Row l (lane l's points) holds 16-byte chunk c
 // at c ^ (l mod 8), |X|^2 rows (64 bytes) at c ^ (l / 2 mod 4): conflict-free on
-// both sides.  Bound by memory: 2^26 points take 183 us (0.88 of the copy rate),
-// as |X|^2 135 us.  (On the tiles of k_block a thread read its points at a stride
+// both sides.  Bound by memory: 2^26 points take 180 us (0.89 of the copy rate),
+// as |X|^2 132 us.  (On the tiles of k_block a thread read its points at a stride
 // of a segment, 32 lanes of n = 16 in one bank pair, and stored them so: n = 16
-// 433 us, |X|^2 330; n = 8 307; n = 4 256.  n = 2 stays there: 176 us against
+// 430 us, |X|^2 327; n = 8 310; n = 4 255.  n = 4 as |X|^2 stays there, see
+// launch_block, and n = 2: 176 us against
 // 182, |X|^2 122 against 134.)
 constexpr int kShortWarps = 8;
 

@@ -92,7 +92,7 @@ cudaError_t launch_fourstep_ws(int log_n, int sign, const FourStepWsArgs &a, cud
 // output): producer warp, three swizzled TMA tile buffers, TMA output stores.
 struct FourStepHwArgs;
 cudaError_t launch_fourstep_hw(int sign, const FourStepHwArgs &a, cudaStream_t st);
-// Lane-line persistent four-step kernel for n = 2^16..2^20 (FP32, complex
+// Lane-line persistent four-step kernel for n = 2^16..2^20 (complex or |X|^2
 // output): lines of 256..1024 points with 32 points per lane, a queue of
 // column and row tiles, a loader warp and a retirer warp per buffer, swizzled TMA tiles.  prec as
 // for launch_block (tensor-core lines at n = 2^16).

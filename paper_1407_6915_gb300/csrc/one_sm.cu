@@ -6,14 +6,16 @@
 //   S1  radix 32 over a from global memory, times w_n^{j k_a}, j = m mod 512
 //   S2  radix 32 over b, times w_512^{c k_b}
 //   S3  radix 16 over c: X[k_a + 32 k_b + 1024 k_c], to global memory
-// Three barriers and 32 bytes of shared-memory traffic per point, and no traffic
-// between SMs.  4001 segments: 186 us (0.84 of the copy rate), against 249 us (0.63)
+// Three barriers and 43 bytes of shared-memory traffic per point (two exchanges,
+// and the rows copied ahead), and no traffic between SMs.  4001 segments: 186 us (0.84 of the copy rate), against 249 us (0.63)
 // for the 4-CTA cluster kernel, which waits for its all-to-all exchange between
 // SMs.  22 of the next segment's 32 rows are copied into the shared memory left
 // over while a segment runs (199 us with all of them read when it starts).  (Four
 // stages of radix 16, 16, 16, 4 with 1024 threads of 64 registers
 // measured 266 us: half as much shared-memory traffic again and a barrier more,
-// and with one CTA per SM nothing overlaps a stage.)
+// and with one CTA per SM nothing overlaps a stage.)  2^15 does not fit an SM; at
+// 2^13 the 2-CTA cluster kernel runs at 0.61 of the copy rate (2000 segments 64
+// us), and this form has not been tried there.
 //
 // Slot of m: m ^ (a mod 16) (8-byte slots).  In S1 and S2 a half-warp takes 16
 // neighbouring m; in S3 16 neighbouring a of one (b, c), so that a warp stores 32

@@ -92,10 +92,10 @@ bool frames_fused(const fftseg_plan_s *p)
 // forward ones on the cluster kernel, and inverse ones there up to n/2 = 2^14
 // for batches of at most 64 MiB of samples.  (The cluster kernel's join reads
 // its bins with plain loads, a point and its mirror:
-// measured on GB300 at n = 2^14 and 2^15 over 4 GiB, 0.37 and 0.35 of the
-// copy peak against 0.39 and 0.37 in 512 MiB chunks, at 256 MiB 0.35 / 0.34
-// against 0.37 / 0.36, and for 37 segments 9.1 / 12.4 us against
-// 12.7 / 14.5 us; from n = 2^16 on it fell to 0.29..0.22, and copying the
+// measured on GB300 at n = 2^14 and 2^15 over 64 MiB of samples, 60 and 56 us
+// against 65 and 62 in 512 MiB chunks, over 256 MiB 218 and 199 against 213 and
+// 191, over 2 GiB 1662 and 1503 against 1628 and 1437; from n = 2^16 on it fell
+// to 0.29..0.22 of the copy peak against 0.35, and copying the
 // bins and their mirrors in ahead by 8-byte cp.async, at two CTAs per SM,
 // measured slower still: 0.33..0.21 at n = 2^14..2^17.)
 bool real_fused(const fftseg_plan_s *p)
@@ -1277,8 +1277,9 @@ int create_real(fftseg_plan *out, int64_t n, int64_t batch, int direction, int n
     p->rchunk = cs;
     unsigned iflags = flags & ~FFTSEG_FLAG_REAL;
     // forward plans of 2^17 samples: the cluster kernel with the split in its
-    // epilogue (one pass) measured 0.39 of the copy peak against 0.36 for the
-    // chunked lane-line transform plus a split pass (at 2^18: 0.28 against 0.35)
+    // epilogue (one pass) takes 1562 us for 2 GiB of samples (0.41 of the copy peak)
+    // against 1662 for the chunked lane-line transform plus a split pass, and 13.5
+    // against 22.7 for 8 MiB (at 2^18 0.28 of the copy peak against 0.35)
     if (direction == FFTSEG_FORWARD && M == (1 << 16) && !(flags & (kPathFlags | FFTSEG_FLAG_AUTOTUNE)))
         iflags |= FFTSEG_FLAG_CLUSTER_LOG2(4);
     int rc = fftseg_plan_create(&p->inner, M, cs, direction, FFTSEG_NORM_NONE, FFTSEG_PREC_FP32,

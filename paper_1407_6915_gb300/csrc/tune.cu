@@ -78,7 +78,7 @@ void append_cache_file(const std::string &key, unsigned flags, double ms)  // wi
 std::vector<unsigned> candidates(int log_n, int prec)
 {
     std::vector<unsigned> c;
-    if (prec != FFTSEG_PREC_FP32 || log_n <= 12) {  // one schedule per size
+    if (prec != FFTSEG_PREC_FP32 || log_n <= 12) {  // one schedule (tensor cores at 2^16: the lane lines, the fastest)
         c.push_back(0);
         return c;
     }
