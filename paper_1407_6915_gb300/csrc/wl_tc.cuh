@@ -38,7 +38,7 @@
 // 1024 segments of 65536 points, FP16 hi+lo: 451 us (BF16: 376 us) against
 // 1159 us on the CTA-tile kernel, whose operands, hi and lo, and results all
 // pass through shared memory once more per stage.  Tensor pipe 37 % active,
-// shared-memory pipe 35 %, issue 35 %: bound by latency, with two compute warps
+// shared-memory pipe 41 %, issue 36 %: bound by latency, with two compute warps
 // per scheduler.  (Sixteen warps, two to four lines: 418 and 410 us, against 439
 // and 377 then.)
 #pragma once
