@@ -145,8 +145,8 @@ __global__ void __launch_bounds__((BlockShape<LOG_L, kFramesLogE<LOG_L>>::T), (B
 // the 32 points of (frame g, k_a), radix 32, and has the bins k_a + A k_b,
 // which go out in runs of A.  Slot of point c of row q = A g + k_a: 32 q + (c ^
 // (q mod 16)), conflict-free on both sides.
-// 100003 frames of 1024 at hop 512, |X|^2: 166 us (0.74 of the copy rate),
-// against 223 us for the tiles of k_block_frames, which spend their time between
+// 100003 frames of 1024 at hop 512, |X|^2: 159 us (0.77 of the copy rate),
+// against 234 us for the tiles of k_block_frames, which spend their time between
 // barriers (three stages and two exchanges of the whole CTA); of 512 at hop 256
 // 0.80.  (Each unit's samples prefetched into L2 a unit ahead measured slower,
 // 170 us: the loads of 16 warps keep the memory busy as it is.)  The samples are

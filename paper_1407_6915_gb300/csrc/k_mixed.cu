@@ -242,15 +242,12 @@ namespace {
 // different slots that share one of the 16 bank pairs.
 int half_warp_wavefronts(const int *slot, int lanes)
 {
-    int most = 0;
+    int count[16] = {}, most = 0;
     for (int i = 0; i < lanes; ++i) {
-        int w = 1;  // different slots in this slot's bank pair, counted from the last one on
-        for (int k = i + 1; k < lanes; ++k) {
-            if (((slot[k] ^ slot[i]) & 15) != 0) continue;
-            bool again = false;
-            for (int l = i; l < k && !again; ++l) again = slot[l] == slot[k];
-            w += !again;
-        }
+        bool again = false;
+        for (int k = 0; k < i && !again; ++k) again = slot[k] == slot[i];
+        if (again) continue;
+        const int w = ++count[slot[i] & 15];
         if (w > most) most = w;
     }
     return most;
@@ -264,33 +261,51 @@ int half_warp_wavefronts(const int *slot, int lanes)
 // butterflies; 379 per thread and stage for the barriers and the start.  (The
 // constant 44 of the fit, the same for all, is left out.)  Tiles of 4096
 // points take 7 % more at equal figures.
-double mixed_cost(int n, const int *radix, int nstages, int tile)
+double stage_cost(int n, int R, int ns, bool last, int tile)
 {
-    const int T = tile / 16, cnt = tile / n;
-    double c = 0;
-    for (int t = 0, ns = 1; t < nstages; ns *= radix[t++]) {
-        const int R = radix[t], m = n / R, nb = cnt * m, passes = (nb + T - 1) / T;
-        int wave = 0, lanes = 0;
-        for (int g0 = 0; g0 < 64 && g0 < nb; g0 += 16) {
-            int in[16], out[16], k = 0;
-            for (; k < 16 && g0 + k < nb; ++k) {
-                const int g = g0 + k, j = g % m, base = g / m * n;
-                in[k] = base + j;
-                out[k] = base + j / ns * ns * R + j % ns;
-            }
-            wave += half_warp_wavefronts(in, k);
-            if (t < nstages - 1) wave += half_warp_wavefronts(out, k);  // (the last stage stores to the output)
-            lanes += k;
+#ifdef FFTSEG_COUNT_STAGE_MODEL
+    FFTSEG_COUNT_STAGE_MODEL;  // (a test counts them)
+#endif
+    const int T = tile / 16, cnt = tile / n, m = n / R, nb = cnt * m, passes = (nb + T - 1) / T;
+    int wave = 0, lanes = 0;
+    for (int g0 = 0; g0 < 64 && g0 < nb; g0 += 16) {
+        int in[16], out[16], k = 0;
+        for (; k < 16 && g0 + k < nb; ++k) {
+            const int g = g0 + k, j = g % m, base = g / m * n;
+            in[k] = base + j;
+            out[k] = base + j / ns * ns * R + j % ns;
         }
-        c += 20.0 * passes * R * T + 12.1 * 16.0 * wave / lanes * R * nb + 379.0 * T;
+        wave += half_warp_wavefronts(in, k);
+        if (!last) wave += half_warp_wavefronts(out, k);  // (the last stage stores to the output)
+        lanes += k;
     }
-    return c / (cnt * (double)n) * (tile == kMixEMax ? 1.07 : 1.0);
+    return 20.0 * passes * R * T + 12.1 * 16.0 * wave / lanes * R * nb + 379.0 * T;
 }
 
 struct MixedBest {
     double cost;
     int tile, radix[kMixMaxStages];
+    // a stage's cost depends on its radix and ns alone (and on being the last, and
+    // the tile): kept by a hash of these, modelled about once each (every schedule
+    // by itself took up to 2.9 ms of a plan's creation, n = 4032, now 0.3)
+    int key[1024];
+    double stage[1024];
 };
+
+double mixed_cost(int n, const int *radix, int nstages, int tile, MixedBest &best)
+{
+    double c = 0;
+    for (int t = 0, ns = 1; t < nstages; ns *= radix[t++]) {
+        const bool last = t == nstages - 1;
+        const int key = ((ns * 32 + radix[t]) * 2 + last) * 2 + (tile == kMixEMax), i = (int)((unsigned)key * 2654435769u >> 22);
+        if (best.key[i] != key) {
+            best.key[i] = key;
+            best.stage[i] = stage_cost(n, radix[t], ns, last, tile);
+        }
+        c += best.stage[i];
+    }
+    return c / (tile / n * (double)n) * (tile == kMixEMax ? 1.07 : 1.0);
+}
 
 // All orders of all factorisations of m into `left` radices, after `depth` of them.
 void mixed_search(int n, int m, int left, int *radix, int depth, MixedBest &best)
@@ -299,7 +314,7 @@ void mixed_search(int n, int m, int left, int *radix, int depth, MixedBest &best
         if (m != 1) return;
         for (int tile = 2048; tile <= kMixEMax; tile *= 2) {
             if (n > tile) continue;
-            const double c = mixed_cost(n, radix, depth, tile);
+            const double c = mixed_cost(n, radix, depth, tile, best);
             if (best.cost > 0 && c >= best.cost) continue;
             best.cost = c;
             best.tile = tile;

@@ -7,7 +7,7 @@
 //   S2  radix 32 over b, times w_512^{c k_b}
 //   S3  radix 16 over c: X[k_a + 32 k_b + 1024 k_c], to global memory
 // Three barriers and 43 bytes of shared-memory traffic per point (two exchanges,
-// and the rows copied ahead), and no traffic between SMs.  4001 segments: 186 us (0.84 of the copy rate), against 249 us (0.63)
+// and the rows copied ahead), and no traffic between SMs.  4001 segments: 181 us (0.87 of the copy rate), against 252 us (0.62)
 // for the 4-CTA cluster kernel, which waits for its all-to-all exchange between
 // SMs.  22 of the next segment's 32 rows are copied into the shared memory left
 // over while a segment runs (199 us with all of them read when it starts).  (Four
