@@ -462,8 +462,8 @@ def tc_split(peak):
             "round_trip_inputs": "uniform seed 3; 32 tones + noise seed 4",
             "bound_fp32_per_transform": "2e-6*log2(n)", "bound_tc_per_transform": 1e-4,
             "role": "accuracy option: the tensor-core forms meet 1e-4 but are slower than FP32 at every size "
-                    "(their operands make a shared-memory round trip per stage on a path whose shared-memory "
-                    "pipe is already the limit)",
+                    "(three products per value; except at 65536 their operands make a shared-memory round "
+                    "trip per stage on a path whose shared-memory pipe is already the limit)",
             "sizes": out}
 
 
